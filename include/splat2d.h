@@ -118,7 +118,8 @@ typedef struct {
  * lowpass sqrt(1/2) px, z_near 0.01, black background. */
 typedef struct {
   int32_t tile_w, tile_h;   /* one of 8x8, 16x16, 32x8 */
-  int32_t chunk;            /* surfels staged per shared-memory batch: 64, 128, 256 (or 512 with 256-pixel tiles) */
+  int32_t chunk;            /* surfels staged per shared-memory batch: 64, 128, 256 (or 512 with 256-pixel tiles); the
+                               forward of 8x8 tiles stages 32 whatever it says */
   float alpha_min;          /* skip pairs with alpha below this */
   float alpha_max;          /* clamp of alpha (keeps the reverse pass finite) */
   float t_min;              /* stop a pixel before T would drop below this */
@@ -141,7 +142,8 @@ typedef struct {
 /* Bits 8..15 of flags: forward tail threshold, pixels per warp of a tile below
  * which the forward shares the tile's remaining pixels across all warps
  * (0 = the default of 6; 255 = always).  A launch-shape knob for the
- * autotuner: it changes the schedule, not the result beyond rounding. */
+ * autotuner: it changes the schedule, not the result beyond rounding.  8x8
+ * tiles are composited by one warp each and ignore it. */
 #define SPLAT2D_FLAG_TAIL_SHIFT 8
 
 /* The shape of one problem: the views (host array) and sizes.  Pass the same
@@ -224,8 +226,8 @@ int splat2d_bin_sort(const splat2d_config* cfg, const splat2d_problem* prob, voi
  * accumulation, I, D, A = sum_i (c_i, z_i, 1) w_i prod_{j<i} (1 - w_j).
  *
  * Forward compositing: one persistent launch over every (view, tile); each
- * tile stages chunks of its sorted surfels in shared memory and composites
- * front to back with warp-level early termination.  Writes rgb, depth,
+ * tile stages chunks of its sorted surfels and composites front to back with
+ * warp-level early termination.  Writes rgb, depth,
  * normal, alpha (packed per view as described above; any may be NULL) and
  * keeps in `ws`, for the backward pass, per-pixel T_final and the last
  * blended index and a copy of every record it staged, in sorted-list order

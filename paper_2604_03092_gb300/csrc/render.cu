@@ -1,26 +1,31 @@
 // Per-tile compositing (forward) and its adjoint (backward).
 //
-// Both kernels are persistent: one CTA per tile-shaped block of pixels pulls
-// (view, tile) work items from an atomic queue ordered longest list first,
-// so many views of uneven size run in one launch.  A tile's sorted surfel
-// list is staged through shared memory in chunks.  For each chunk every lane
-// (one pixel) gets a bitmask of the chunk entries whose pixel rect holds its
-// pixel, built with 12 ballots per 32 entries (which entries span each column
-// and each row of the warp's 8x4 patch), and then walks only its own entries:
-// surfels are a few pixels wide, so a lane-per-pixel walk over a shared entry
-// sequence would leave most lanes idle, while here nearly every lane does a
-// useful (pixel, surfel) evaluation on every step.
+// All kernels are persistent: CTAs (16x16 and 32x8 tiles) or warps (8x8
+// tiles) pull (view, tile) work items from an atomic queue ordered longest
+// list first, so many views of uneven size run in one launch.
 //
 // Forward (Eq. 1): front to back per pixel, alpha = min(alpha_max, sigma*G),
 // pairs below alpha_min skipped, stop before T would fall below t_min; the
 // tile stops staging as soon as all its pixels have stopped.
 // Backward: back to front per pixel from its last blended entry, T recovered
 // by division, one scalar suffix sum per pixel (the upstream gradient dotted
-// with the features of the entries behind), evaluated 32 (pixel, entry) pairs
-// at a time with segmented warp scans; each lane adds its pair's gradient to
-// the entry's shared-memory slot, and after the chunk one set of vector
-// atomics per (tile, entry) moves the sums to the gradient record.
+// with the features of the entries behind).
+//
+// Forward, 8x8 tiles (the shape the autotuner keeps): one warp per tile, see
+// k_render_fwd_warp.
+//
+// Forward of 256-pixel tiles, and backward: one CTA per tile.  The sorted surfel list is staged
+// through shared memory in chunks; for each chunk every lane (one pixel) gets
+// a bitmask of the chunk entries whose pixel rect holds its pixel, built with
+// 12 ballots per 32 entries (which entries span each column and each row of
+// the warp's 8x4 patch), and walks its own entries.  The backward evaluates 32
+// (pixel, entry) pairs at a time with segmented warp scans; each lane adds its
+// pair's gradient to the entry's shared-memory slot, and after the chunk one
+// set of vector atomics per (tile, entry) moves the sums to the gradient
+// record.
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "splat2d_internal.cuh"
 
@@ -94,6 +99,71 @@ __device__ __forceinline__ void eval_pair(const float4 c, const float4 p, const 
   const float raw = __fmul_rn(q.w, e.G);
   e.clamped = raw > alpha_max;
   e.alpha = e.clamped ? alpha_max : raw;
+}
+
+// Two floats in one 64-bit register pair: one instruction operates on both
+// (sm_100's packed FP32), each half rounded like the scalar operation.
+struct F2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ F2 pk2(float lo, float hi) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ F2 pk2(float x) { return pk2(x, x); }
+__device__ __forceinline__ float2 f2_get(F2 a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+  return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 f2_sub(F2 a, F2 b) {
+  F2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+
+// eval_pair of one record at two pixels, bit for bit.
+struct Pair2 {
+  float alpha[2], rc[2];
+  bool obj[2], clamped[2];
+};
+__device__ __forceinline__ void eval_pair2(const float4 c, const float4 p, const float4 q, F2 px, F2 py,
+                                           float lp_scale, float alpha_max, Pair2& e) {
+  const F2 dx = f2_sub(f2_sub(px, pk2(c.x)), pk2(c.z));
+  const F2 dy = f2_sub(f2_sub(py, pk2(c.y)), pk2(c.w));
+  const F2 a = f2_fma(pk2(p.x), dx, f2_mul(pk2(p.y), dy));
+  const F2 b = f2_fma(pk2(p.z), dx, f2_mul(pk2(p.w), dy));
+  const float2 cc = f2_get(f2_fma(pk2(q.x), dx, f2_fma(pk2(q.y), dy, pk2(q.z))));
+  e.rc[0] = rcp_approx(cc.x);
+  e.rc[1] = rcp_approx(cc.y);
+  const F2 rc = pk2(e.rc[0], e.rc[1]);
+  const F2 ua = f2_mul(a, rc), vb = f2_mul(b, rc);
+  const float2 ro = f2_get(f2_fma(ua, ua, f2_mul(vb, vb)));
+  const float2 rl = f2_get(f2_mul(pk2(lp_scale), f2_fma(dx, dx, f2_mul(dy, dy))));
+  e.obj[0] = ro.x <= rl.x;
+  e.obj[1] = ro.y <= rl.y;
+  const float G0 = ex2_approx(-(e.obj[0] ? ro.x : rl.x)), G1 = ex2_approx(-(e.obj[1] ? ro.y : rl.y));
+  const float2 raw = f2_get(f2_mul(pk2(q.w), pk2(G0, G1)));
+  e.clamped[0] = raw.x > alpha_max;
+  e.clamped[1] = raw.y > alpha_max;
+  e.alpha[0] = e.clamped[0] ? alpha_max : raw.x;
+  e.alpha[1] = e.clamped[1] ? alpha_max : raw.y;
 }
 
 // Depth a pair contributes to the depth output: the center's depth z
@@ -324,7 +394,7 @@ struct FwdSmem {
 // back: each blended pair adds 2 w (z A - D) with A = 1 - T and D the depth
 // sum in front of it).
 template <int TW, int TH, int CHUNK, bool DIST>
-__global__ void __launch_bounds__(TW* TH, (TW * TH == 64) ? (CHUNK <= 64 ? 16 : 12) : 3) k_render_fwd(const RenderArgs A) {
+__global__ void __launch_bounds__(TW* TH, 3) k_render_fwd(const RenderArgs A) {
   constexpr int NT = TW * TH, NW = NT / 32, WX = TW / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   FwdSmem<NT, CHUNK>& S = *reinterpret_cast<FwdSmem<NT, CHUNK>*>(smem_raw);
@@ -561,6 +631,390 @@ __global__ void __launch_bounds__(TW* TH, (TW * TH == 64) ? (CHUNK <= 64 ? 16 : 
     if (lane == 0) {
       atomicAdd(&A.hdr->stat[STAT_FWD_EVAL], a);
       atomicAdd(&A.hdr->stat[STAT_FWD_BLEND], bb);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Forward for 8x8 tiles
+// ---------------------------------------------------------------------------
+// One warp per tile (NP = 2), or per half of a tile (NP = 1: four rows; where
+// there are too few tiles to fill the GPU), no block barriers.  The tile's
+// list is taken 32 entries at a time, in two passes:
+//   1. entry-major: each lane owns an entry, its record in registers, and
+//      evaluates alpha at the active pixels of its rect (a bit mask), two per
+//      step in packed FP32; alphas of at least alpha_min go to a pixel x entry
+//      table in shared memory and set a bit in the entry's pixel mask;
+//   2. pixel-major: the masks are transposed across the warp, each lane owns
+//      NP pixels and blends their set bits front to back.
+// Against a walk in which each lane evaluates and blends its own pixel's
+// entries from a chunk staged in shared memory (k_render_fwd): a surfel's
+// pixels in the tile are more even in number than the entries of a pixel,
+// which the depth order concentrates in a band of the tile; the evaluation
+// reads no shared memory; and the pairs below alpha_min (40% of them) never
+// reach the pass that blends: 6.9 warp instructions per evaluated pair against
+// 10.2.  A chunk whose rects cover a third of the pixels or more is walked by
+// all lanes together instead.
+// Issue-bound (71% of the issue slots on 4 keyframes x 4 views); the blending
+// pass keeps 17% of its lanes busy where many keyframes overlap, 41% on one.
+// 24 keyframes x 24 views at 512x384: 16.3 -> 11.0 ms; one keyframe x 8 views
+// 557 -> 440 us.
+constexpr int WARPS = 4;       // warps per CTA of the warp-per-tile kernels; they share nothing
+constexpr int FW_STRIDE = 33;  // floats per pixel row of the alpha table
+// (pixel, entry) pairs per 32 pixels (of 1024) that make a chunk dense: two
+// 333x251 views of 20 K large surfels 157 us without the dense walk, 129 with
+// it; 275 and 450 were slower on keyframes.
+constexpr uint32_t FW_DENSE = 350;
+// Up to this many tiles per SM a warp takes half a tile: twice the warps, and
+// a shorter chain per chunk, where the tiles are too few for whole ones to
+// keep the SM's 24 warps busy.  Whole against half, 8 keyframes in one view:
+// 300 tiles 1319 / 921 us, 1900 tiles 365 / 290, 3072 tiles 344 / 293; one
+// keyframe, 3072 tiles 83 / 88; 7260 tiles 317 / 308; 24576 tiles 440 / 499.
+constexpr int FW_WHOLE_TILES_PER_SM = 32;
+
+template <int NP>
+struct FwdWarpBase {
+  float alpha[32 * NP * FW_STRIDE];  // [pixel][entry]; RAY: negative where the object-space term decides
+  float4 col[32];                    // r g b z
+  float4 nrm[32];                    // nx ny nz p22
+};
+template <int NP>
+struct FwdWarpRay : FwdWarpBase<NP> {
+  float4 c[32];  // cx_hi cy_hi cx_lo cy_lo
+  float2 q[32];  // p20 p21
+};
+template <int NP, bool RAY>
+using FwdWarpSmem = std::conditional_t<RAY, FwdWarpRay<NP>, FwdWarpBase<NP>>;
+
+// Transpose of the 32x32 bit matrix whose row i is lane i's word: lane i
+// returns column i (bit k = bit i of lane k's word).
+__device__ __forceinline__ uint32_t warp_transpose_bits(uint32_t x, int lane) {
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    // m: the bits of each 2s-group that stay in the lower lane
+    const uint32_t m = s == 16 ? 0x0000ffffu : s == 8 ? 0x00ff00ffu : s == 4 ? 0x0f0f0f0fu : s == 2 ? 0x33333333u
+                                                                                                   : 0x55555555u;
+    const bool upper = lane & s;
+    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, s);
+    const uint32_t keep = upper ? ~m : m;
+    x = (x & keep) | (__funnelshift_l(y, y, upper ? 32 - s : s) & ~keep);
+  }
+  return x;
+}
+
+// The pixels of an 8x4 block at (x0, y0) (bit y * 8 + x) inside a record's
+// pixel rect, given as (x0 | y0 << 16, x1 | y1 << 16), inclusive.
+__device__ __forceinline__ uint32_t block_rect_mask(uint32_t r0, uint32_t r1, int x0, int y0) {
+  const int a0 = max((int)(r0 & 0xffffu) - x0, 0), a1 = min((int)(r1 & 0xffffu) - x0, 7);
+  const int b0 = max((int)(r0 >> 16) - y0, 0), b1 = min((int)(r1 >> 16) - y0, 3);
+  if (a0 > a1 || b0 > b1) return 0u;
+  const uint32_t row = ((2u << a1) - 1u) & ~((1u << a0) - 1u);
+  return (row * 0x01010101u) & (0xffffffffu << (8 * b0)) & (0xffffffffu >> (8 * (3 - b1)));
+}
+
+// The next two pixels of an entry's masks (the same one twice, two = false,
+// where its current word has only one left), taken out of them.
+template <int NP>
+struct PixelStep {
+  int pix[2];        // pixel numbers, 32 * word + bit
+  uint32_t bit[2];
+  bool second_word;  // the word they came from
+  bool two;
+  __device__ __forceinline__ explicit PixelStep(uint32_t (&m)[NP]) {
+    second_word = NP == 2 && m[0] == 0u;
+    const uint32_t cur = NP == 2 && second_word ? m[NP - 1] : m[0];
+    bit[0] = cur & (0u - cur);
+    const uint32_t rest = cur ^ bit[0];
+    two = rest != 0u;
+    bit[1] = two ? rest & (0u - rest) : bit[0];
+    const int off = second_word ? 32 : 0;
+    pix[0] = 31 - __clz(bit[0]) + off;
+    pix[1] = 31 - __clz(bit[1]) + off;
+    const uint32_t left = rest & (rest - 1);
+    if (NP == 2 && second_word) m[NP - 1] = left;
+    else m[0] = left;
+  }
+};
+template <int NP>
+__device__ __forceinline__ uint32_t count_bits(const uint32_t (&m)[NP]) {
+  return NP == 2 ? __popc(m[0]) + __popc(m[NP - 1]) : __popc(m[0]);
+}
+template <int NP>
+__device__ __forceinline__ bool any_bits(const uint32_t (&m)[NP]) {
+  return (m[0] | m[NP - 1]) != 0u;
+}
+
+// One pixel's compositing state.
+template <bool DIST>
+struct PixelSums {
+  float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f, D = 0.f, N0 = 0.f, N1 = 0.f, N2 = 0.f, Ds = 0.f;
+  // adds an entry of weight w (T: the transmittance in front of it)
+  __device__ __forceinline__ void add(float w, float r, float g, float b, float z, float nx, float ny, float nz) {
+    C0 = __fmaf_rn(w, r, C0);
+    C1 = __fmaf_rn(w, g, C1);
+    C2 = __fmaf_rn(w, b, C2);
+    if constexpr (DIST) Ds = __fmaf_rn(2.f * w, __fmaf_rn(z, __fsub_rn(1.f, T), -D), Ds);
+    D = __fmaf_rn(w, z, D);
+    N0 = __fmaf_rn(w, nx, N0);
+    N1 = __fmaf_rn(w, ny, N1);
+    N2 = __fmaf_rn(w, nz, N2);
+  }
+};
+
+// Blends the entries of `todo` (ascending) into one pixel; returns those
+// blended (all, or those before the first that would take T below t_min).
+template <int NP, bool RAY, bool DIST>
+__device__ __forceinline__ uint32_t blend_pixel(const FwdWarpSmem<NP, RAY>& S, int pix, uint32_t todo, float px,
+                                                float py, float t_min, PixelSums<DIST>& s, bool& done) {
+  uint32_t k = todo;
+  while (k) {
+    const int e = __ffs(k) - 1;
+    const float av = S.alpha[pix * FW_STRIDE + e];
+    const float alpha = RAY ? fabsf(av) : av;
+    const float Tn = __fmul_rn(s.T, __fsub_rn(1.f, alpha));
+    if (Tn < t_min) {
+      done = true;
+      return todo & ((1u << e) - 1u);
+    }
+    k &= k - 1;
+    const float w = __fmul_rn(alpha, s.T);
+    const float4 col = S.col[e], nrm = S.nrm[e];
+    float zp = col.w;
+    if constexpr (RAY) {
+      // depth of the ray-splat intersection (see pair_depth): the same c as eval_pair's
+      const float4 c = S.c[e];
+      const float2 q = S.q[e];
+      const float dx = __fsub_rn(__fsub_rn(px, c.x), c.z), dy = __fsub_rn(__fsub_rn(py, c.y), c.w);
+      const float rc = rcp_approx(__fmaf_rn(q.x, dx, __fmaf_rn(q.y, dy, nrm.w)));
+      if (__float_as_int(av) < 0) zp = col.w * nrm.w * rc;
+    }
+    s.add(w, col.x, col.y, col.z, zp, nrm.x, nrm.y, nrm.z);
+    s.T = Tn;
+  }
+  return todo;
+}
+
+// 80 registers: 6 CTAs (24 warps) per SM, as many as the alpha tables leave
+// room for (NP = 2).
+template <int NP, bool RAY, bool DIST>
+__global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(const RenderArgs A) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  FwdWarpSmem<NP, RAY>& S = reinterpret_cast<FwdWarpSmem<NP, RAY>*>(smem_raw)[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const RastParams& P = A.P;
+  uint32_t n_eval = 0, n_blend = 0;
+  // a failed binning (instance capacity exceeded) leaves no valid lists
+  if (A.hdr->status != 0) return;
+  for (;;) {
+    uint32_t item = 0;
+    if (lane == 0) item = atomicAdd(&A.hdr->queue_fwd, 1u);
+    item = __shfl_sync(0xffffffffu, item, 0);
+    const int half = NP == 1 ? (int)(item & 1u) : 0;
+    if (NP == 1) item >>= 1;
+    if ((int64_t)item >= A.T) break;
+    const int t = (int)__ldg(A.order + item);
+    const int v = find_view_by_tile(A.views, A.V, t);
+    const DView& vw = A.views[v];
+    const int lt = t - vw.tile_base;
+    const int tx0 = (lt % vw.tiles_x) * 8, ty0 = (lt / vw.tiles_x) * 8 + 4 * half;
+    const float fx0 = (float)tx0 + 0.5f, fy0 = (float)ty0 + 0.5f;
+    // this lane's pixels: row lane / 8, and with NP = 2 the one four rows below
+    const int ipx = tx0 + (lane & 7), ipy = ty0 + (lane >> 3);
+    const float px = (float)ipx + 0.5f, py0 = (float)ipy + 0.5f, py1 = (float)(ipy + 4) + 0.5f;
+    const uint2 range = __ldg(A.ranges + t);
+    PixelSums<DIST> ps[NP];
+    uint32_t last[NP];
+    bool done[NP];
+#pragma unroll
+    for (int h = 0; h < NP; h++) {
+      last[h] = range.x;
+      done[h] = !(ipx < vw.W && ipy + 4 * h < vw.H);
+    }
+    // this lane's list entry of the chunk staged next, read one chunk ahead
+    uint32_t ent = range.x + lane < range.y ? __ldg(A.vals + range.x + lane) : 0u;
+    uint32_t word = (range.x >> 5) + (uint32_t)t;  // the chunk's blended-mask word
+    for (int64_t base = range.x; base < range.y; base += 32, word++) {
+      uint32_t live_px[NP];
+#pragma unroll
+      for (int h = 0; h < NP; h++) live_px[h] = __ballot_sync(0xffffffffu, !done[h]);
+      if (!any_bits<NP>(live_px)) break;
+      const int count = (int)min64(32, (int64_t)range.y - base);
+      const uint32_t sf = ent;
+      ent = base + 32 + lane < (int64_t)range.y ? __ldg(A.vals + base + 32 + lane) : 0u;
+      const bool ok =
+          lane < count && s2d_check((int64_t)sf >= vw.soff && (int64_t)sf < vw.soff + vw.scnt, A.hdr);
+      const uint32_t ri = ok ? (uint32_t)(vw.rbase + ((int64_t)sf - vw.soff)) : 0xffffffffu;
+      // gather the chunk's records: five neighbouring lanes take one record's
+      // five float4, so a load instruction touches the lines of seven records
+      // (a lane per record touches 32, five times over: that bound the gather
+      // on L1 tag lookups) and a store to the sorted-order copy is contiguous
+      float4* raw = reinterpret_cast<float4*>(S.alpha);  // until pass 1 writes alphas there
+      {
+        float4 f[REC_F4];
+#pragma unroll
+        for (int k = 0; k < REC_F4; k++) {
+          const int i = lane + 32 * k, e = (i * 205) >> 10;  // i / 5 for i < 160
+          const uint32_t r = __shfl_sync(0xffffffffu, ri, e);
+          f[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (r != 0xffffffffu) f[k] = __ldg(A.records + (size_t)r * REC_F4 + (i - 5 * e));
+        }
+#pragma unroll
+        for (int k = 0; k < REC_F4; k++) {
+          const int i = lane + 32 * k;
+          raw[i] = f[k];
+          // the backward reads the records in list order; streaming stores, read long after
+          if (i < count * REC_F4) __stcs(A.rcopy + base * REC_F4 + i, f[k]);
+        }
+      }
+      __syncwarp();
+      float4 c = make_float4(0.f, 0.f, 0.f, 0.f), p = c, q = c;
+      uint32_t m[NP];  // active pixels in the entry's rect
+#pragma unroll
+      for (int h = 0; h < NP; h++) m[h] = 0u;
+      if (ok) {
+        const float4 f0 = raw[lane * REC_F4], f1 = raw[lane * REC_F4 + 1], f2 = raw[lane * REC_F4 + 2],
+                     f3 = raw[lane * REC_F4 + 3], f4 = raw[lane * REC_F4 + 4];
+        const float2 cl = unpack_half2_scaled(__float_as_uint(f0.z));
+        c = make_float4(f0.x, f0.y, cl.x, cl.y);
+        p = f1;
+        q = make_float4(f2.x, f2.y, f2.z, f0.w);
+        S.col[lane] = make_float4(f2.w, f3.x, f3.y, f4.y);
+        S.nrm[lane] = make_float4(f3.z, f3.w, f4.x, f2.z);
+        if constexpr (RAY) {
+          S.c[lane] = c;
+          S.q[lane] = make_float2(f2.x, f2.y);
+        }
+#pragma unroll
+        for (int h = 0; h < NP; h++)
+          m[h] = block_rect_mask(__float_as_uint(f4.z), __float_as_uint(f4.w), tx0, ty0 + 4 * h) & live_px[h];
+      }
+      __syncwarp();
+      const uint32_t pairs = count_bits<NP>(m);
+      n_eval += pairs;
+      uint32_t bl[NP];  // entries blended at this lane's pixels
+#pragma unroll
+      for (int h = 0; h < NP; h++) bl[h] = 0u;
+      if (__reduce_add_sync(0xffffffffu, pairs) >= FW_DENSE * NP) {
+        // ---- dense chunk: every lane walks every entry at its pixels -----------
+#pragma unroll 2
+        for (int e = 0; e < count; e++) {
+          const float4* rec = raw + e * REC_F4;
+          const float4 f0 = rec[0], f1 = rec[1], f2 = rec[2], f3 = rec[3], f4 = rec[4];
+          const float2 cl = unpack_half2_scaled(__float_as_uint(f0.z));
+          Pair2 pr;
+          eval_pair2(make_float4(f0.x, f0.y, cl.x, cl.y), f1, make_float4(f2.x, f2.y, f2.z, f0.w), pk2(px),
+                     pk2(py0, py1), P.lp_scale, P.alpha_max, pr);
+#pragma unroll
+          for (int h = 0; h < NP; h++) {
+            const uint32_t on = (__shfl_sync(0xffffffffu, m[h], e) >> lane) & 1u;
+            if (!on || done[h] || pr.alpha[h] < P.alpha_min) continue;
+            const float Tn = __fmul_rn(ps[h].T, __fsub_rn(1.f, pr.alpha[h]));
+            if (Tn < P.t_min) {
+              done[h] = true;
+              continue;
+            }
+            const float zp = RAY && pr.obj[h] ? f4.y * f2.z * pr.rc[h] : f4.y;  // see pair_depth
+            ps[h].add(__fmul_rn(pr.alpha[h], ps[h].T), f2.w, f3.x, f3.y, zp, f3.z, f3.w, f4.x);
+            ps[h].T = Tn;
+            bl[h] |= 1u << e;
+          }
+        }
+      } else {
+        // ---- pass 1: alphas, an entry per lane ---------------------------------
+        uint32_t kept[NP];  // pixels where this entry's alpha is at least alpha_min
+#pragma unroll
+        for (int h = 0; h < NP; h++) kept[h] = 0u;
+        uint32_t live;
+        while ((live = __ballot_sync(0xffffffffu, any_bits<NP>(m))) != 0u) {
+          // a few long lists left: the warp takes them pixel by lane instead
+          // (about 80 instructions per entry, against 75 per step of two pixels)
+          const int nl = __popc(live);
+          if (nl <= 8 && 2 * (int)__reduce_max_sync(0xffffffffu, count_bits<NP>(m)) > 3 * nl + 1) break;
+          if (any_bits<NP>(m)) {
+            const PixelStep<NP> st(m);
+            Pair2 e;
+            eval_pair2(c, p, q, f2_add(pk2(fx0), pk2((float)(st.pix[0] & 7), (float)(st.pix[1] & 7))),
+                       f2_add(pk2(fy0), pk2((float)(st.pix[0] >> 3), (float)(st.pix[1] >> 3))), P.lp_scale,
+                       P.alpha_max, e);
+            const uint32_t k = (e.alpha[0] < P.alpha_min ? 0u : st.bit[0]) | (e.alpha[1] < P.alpha_min ? 0u : st.bit[1]);
+#pragma unroll
+            for (int i = 0; i < 2; i++)
+              S.alpha[st.pix[i] * FW_STRIDE + lane] = RAY && e.obj[i] ? -e.alpha[i] : e.alpha[i];
+            if (NP == 2 && st.second_word) kept[NP - 1] |= k;
+            else kept[0] |= k;
+          }
+        }
+        while (live) {
+          const int src = __ffs(live) - 1;
+          live &= live - 1;
+          auto from = [&](float x) { return __shfl_sync(0xffffffffu, x, src); };
+          const float4 ec = make_float4(from(c.x), from(c.y), from(c.z), from(c.w));
+          const float4 ep = make_float4(from(p.x), from(p.y), from(p.z), from(p.w));
+          const float4 eq = make_float4(from(q.x), from(q.y), from(q.z), from(q.w));
+          Pair2 e;
+          eval_pair2(ec, ep, eq, pk2(px), pk2(py0, py1), P.lp_scale, P.alpha_max, e);
+#pragma unroll
+          for (int h = 0; h < NP; h++) {
+            const bool on = (__shfl_sync(0xffffffffu, m[h], src) >> lane) & 1u;
+            if (on) S.alpha[(lane + 32 * h) * FW_STRIDE + src] = RAY && e.obj[h] ? -e.alpha[h] : e.alpha[h];
+            const uint32_t k = __ballot_sync(0xffffffffu, on && !(e.alpha[h] < P.alpha_min));
+            if (lane == src) kept[h] |= k;
+          }
+        }
+        // ---- pass 2: blending, NP pixels per lane ------------------------------
+        uint32_t todo[NP];
+#pragma unroll
+        for (int h = 0; h < NP; h++) todo[h] = warp_transpose_bits(kept[h], lane);
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < NP; h++)
+          bl[h] = blend_pixel<NP, RAY, DIST>(S, lane + 32 * h, todo[h], px, h ? py1 : py0, P.t_min, ps[h], done[h]);
+      }
+#pragma unroll
+      for (int h = 0; h < NP; h++) {
+        if (bl[h]) last[h] = (uint32_t)base + 32u - __clz(bl[h]);
+        n_blend += __popc(bl[h]);
+        // streaming stores: read once, by the backward, long after
+        if (s2d_check((int64_t)word < A.bmask_words, A.hdr))
+          __stcs(A.bmask + (size_t)word * 64 + 32 * (half + h) + lane, bl[h]);
+      }
+      __syncwarp();
+    }
+    const int64_t HW = (int64_t)vw.W * vw.H;
+#pragma unroll
+    for (int h = 0; h < NP; h++) {
+      if (!(ipx < vw.W && ipy + 4 * h < vw.H)) continue;
+      const PixelSums<DIST>& s = ps[h];
+      const int64_t pix = (int64_t)(ipy + 4 * h) * vw.W + ipx;
+      if (A.rgb) {
+        float* o = A.rgb + 3 * vw.poff + pix;
+        o[0] = __fmaf_rn(s.T, P.bg[0], s.C0);
+        o[HW] = __fmaf_rn(s.T, P.bg[1], s.C1);
+        o[2 * HW] = __fmaf_rn(s.T, P.bg[2], s.C2);
+      }
+      if (A.depth) A.depth[vw.poff + pix] = s.D;
+      if (A.normal) {
+        float* o = A.normal + 3 * vw.poff + pix;
+        o[0] = s.N0;
+        o[HW] = s.N1;
+        o[2 * HW] = s.N2;
+      }
+      if (A.alpha) A.alpha[vw.poff + pix] = 1.f - s.T;
+      if constexpr (DIST) A.dist[vw.poff + pix] = s.Ds;
+      A.tfinal[vw.poff + pix] = s.T;
+      A.last[vw.poff + pix] = last[h];
+      A.dfinal[vw.poff + pix] = s.D;
+    }
+  }
+  if (P.stats) {
+    unsigned long long a = n_eval, b = n_blend;
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if (lane == 0) {
+      atomicAdd(&A.hdr->stat[STAT_FWD_EVAL], a);
+      atomicAdd(&A.hdr->stat[STAT_FWD_BLEND], b);
     }
   }
 }
@@ -1179,6 +1633,31 @@ static cudaError_t run_fwd_k(const RenderArgs& A, cudaStream_t st) {
   count_launches(1);
   return cudaGetLastError();
 }
+// One warp-per-tile launch: NP = 2 pixels per lane, or 1 (two items per tile).
+template <int NP, typename K>
+static cudaError_t run_warp_kernel(K k, size_t smem, const RenderArgs& A, int64_t& grid_T, int& grid, cudaStream_t st) {
+  const int64_t items = NP == 2 ? A.T : 2 * A.T;
+  if (grid < 0) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (grid < 0 || grid_T != A.T) {
+    grid = persistent_grid(k, WARPS * 32, smem, (items + WARPS - 1) / WARPS);
+    grid_T = A.T;
+  }
+  k<<<grid, WARPS * 32, smem, st>>>(A);
+  count_launches(1);
+  return cudaGetLastError();
+}
+template <int NP, bool RAY, bool DIST>
+static cudaError_t run_fwd_warp(const RenderArgs& A, cudaStream_t st) {
+  static int grid = -1;
+  static int64_t grid_T = -1;
+  return run_warp_kernel<NP>(k_render_fwd_warp<NP, RAY, DIST>, sizeof(FwdWarpSmem<NP, RAY>) * WARPS, A, grid_T, grid,
+                             st);
+}
+template <int NP>
+static cudaError_t run_fwd_tiles8(const RenderArgs& A, cudaStream_t st) {
+  if (A.P.depth_ray) return A.dist ? run_fwd_warp<NP, true, true>(A, st) : run_fwd_warp<NP, true, false>(A, st);
+  return A.dist ? run_fwd_warp<NP, false, true>(A, st) : run_fwd_warp<NP, false, false>(A, st);
+}
 template <int TW, int TH, int CHUNK>
 static cudaError_t run_fwd(const RenderArgs& A, cudaStream_t st) {
   return A.dist ? run_fwd_k<TW, TH, CHUNK, true>(A, st) : run_fwd_k<TW, TH, CHUNK, false>(A, st);
@@ -1217,6 +1696,7 @@ static cudaError_t run_max_error(const RenderArgs& A, const float* err, uint32_t
   return cudaGetLastError();
 }
 
+// The 256-pixel tile shapes.
 #define S2D_DISPATCH(FN, TWv, THv, CH, ...)                                   \
   do {                                                                        \
     if (TWv == 16 && THv == 16) {                                             \
@@ -1224,10 +1704,6 @@ static cudaError_t run_max_error(const RenderArgs& A, const float* err, uint32_t
       if (CH == 128) return FN<16, 16, 128>(__VA_ARGS__);                     \
       if (CH == 256) return FN<16, 16, 256>(__VA_ARGS__);                     \
       if (CH == 512) return FN<16, 16, 512>(__VA_ARGS__);                     \
-    } else if (TWv == 8 && THv == 8) {                                        \
-      if (CH == 64) return FN<8, 8, 64>(__VA_ARGS__);                         \
-      if (CH == 128) return FN<8, 8, 128>(__VA_ARGS__);                       \
-      if (CH == 256) return FN<8, 8, 256>(__VA_ARGS__);                       \
     } else if (TWv == 32 && THv == 8) {                                       \
       if (CH == 64) return FN<32, 8, 64>(__VA_ARGS__);                        \
       if (CH == 128) return FN<32, 8, 128>(__VA_ARGS__);                      \
@@ -1249,6 +1725,8 @@ cudaError_t launch_render_fwd(const Layout& L, const RastParams& P, int chunk, c
   Header* hdr = reinterpret_cast<Header*>(ws + L.header);
   cudaError_t e = cudaMemsetAsync(&hdr->queue_fwd, 0, sizeof(uint32_t), st);
   if (e != cudaSuccess) return e;
+  if (P.tile_w == 8 && P.tile_h == 8)
+    return A.T > (int64_t)FW_WHOLE_TILES_PER_SM * sm_count() ? run_fwd_tiles8<2>(A, st) : run_fwd_tiles8<1>(A, st);
   S2D_DISPATCH(run_fwd, P.tile_w, P.tile_h, chunk, A, st);
 }
 
@@ -1265,6 +1743,12 @@ cudaError_t launch_render_bwd(const Layout& L, const RastParams& P, int chunk, c
   Header* hdr = reinterpret_cast<Header*>(ws + L.header);
   cudaError_t e = cudaMemsetAsync(&hdr->queue_bwd, 0, sizeof(uint32_t), st);
   if (e != cudaSuccess) return e;
+  if (P.tile_w == 8 && P.tile_h == 8) {
+    if (chunk == 64) return run_bwd<8, 8, 64>(A, st);
+    if (chunk == 128) return run_bwd<8, 8, 128>(A, st);
+    if (chunk == 256) return run_bwd<8, 8, 256>(A, st);
+    return cudaErrorInvalidValue;
+  }
   S2D_DISPATCH(run_bwd, P.tile_w, P.tile_h, chunk, A, st);
 }
 
