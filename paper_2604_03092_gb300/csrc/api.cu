@@ -71,7 +71,7 @@ static bool build_tables(const splat2d_config* cfg, const splat2d_problem* prob,
     H->views.assign(V, DView{});
     H->groups.clear();
   }
-  int64_t R = 0, T = 0, P = 0, work = 0;
+  int64_t R = 0, T = 0, P = 0, work = 0, longest = 0;
   int G = 0;
   std::vector<std::pair<int64_t, int64_t>> ranges;
   for (int v = 0; v < V; v++) {
@@ -124,6 +124,7 @@ static bool build_tables(const splat2d_config* cfg, const splat2d_problem* prob,
       d.group = G - 1;
     }
     R += sv.surfel_count;
+    longest = std::max<int64_t>(longest, sv.surfel_count);
     T += (int64_t)tx * ty;
     P = std::max<int64_t>(P, sv.pixel_offset + (int64_t)sv.width * sv.height);
   }
@@ -140,6 +141,7 @@ static bool build_tables(const splat2d_config* cfg, const splat2d_problem* prob,
   L->P = P;
   L->cap = prob->instance_capacity;
   L->n_work = work;
+  L->max_range = longest;
   L->groups_overlap = overlap;
   L->sort_blocks = std::min(SORT_MAX_BLOCKS, 4 * sm_count());
   L->key_bits = key_bits_for(T);
@@ -162,10 +164,10 @@ static bool build_tables(const splat2d_config* cfg, const splat2d_problem* prob,
   L->vals1 = take(sizeof(uint32_t) * L->cap);
   L->sort_hist = take(sizeof(uint32_t) * (256 * (size_t)L->sort_blocks + 256));
   L->ranges = take(sizeof(uint2) * T);
-  L->tile_count = take(sizeof(uint32_t) * T);   // instances per tile (counted by the preprocess)
+  L->tile_count = take(sizeof(uint32_t) * T);   // instances per tile (zero between binnings)
   L->tile_cursor = take(sizeof(uint32_t) * T);  // scatter cursors (from the tile scan)
   L->tile_order = take(sizeof(uint32_t) * T);
-  L->tile_hist = take(sizeof(uint32_t) * (ORDER_BINS + 16));
+  L->tile_hist = take(sizeof(uint32_t) * TILE_HIST_WORDS);
   L->tile_class = take(sizeof(uint32_t) * 6 * (size_t)T);  // one list per bucket-sort size class
   L->tfinal = take(sizeof(float) * P);
   L->last = take(sizeof(uint32_t) * P);
@@ -276,12 +278,13 @@ int splat2d_preprocess(const splat2d_config* cfg, const splat2d_problem* prob, c
   build_tables(cfg, prob, &L, &H);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
-  if (cudaMemsetAsync(w + L.header, 0, 256, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
-  if (launch_upload(H.views.data(), sizeof(DView) * H.views.size(), w + L.views, st) != cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
-  if (!H.groups.empty() &&
-      launch_upload(H.groups.data(), sizeof(DGroup) * H.groups.size(), w + L.groups, st) != cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
+  // the header (zero), the views and the groups as they lie in the workspace
+  const size_t table_bytes = L.groups + sizeof(DGroup) * H.groups.size() - L.header;
+  std::vector<char> tables(table_bytes, 0);
+  std::memcpy(tables.data() + (L.views - L.header), H.views.data(), sizeof(DView) * H.views.size());
+  if (!H.groups.empty())
+    std::memcpy(tables.data() + (L.groups - L.header), H.groups.data(), sizeof(DGroup) * H.groups.size());
+  if (launch_setup(tables.data(), table_bytes, L, w, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
   RastParams P = make_params(cfg);
   if (launch_preprocess(surfels, L, P, w, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
   return SPLAT2D_OK;
@@ -296,7 +299,6 @@ int splat2d_bin_sort(const splat2d_config* cfg, const splat2d_problem* prob, voi
   char* w = static_cast<char*>(ws);
   RastParams P = make_params(cfg);
   if (launch_bin_tiles(L, P, w, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
-  if (launch_order(L, w, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
   return SPLAT2D_OK;
 }
 

@@ -45,7 +45,92 @@ struct TileBinArgs {
   unsigned long long* bucket;
   int64_t cap;        // instance capacity (bucket length)
   Header* hdr;
+  // scatter pass: the tiles' size classes and work-order bins
+  const uint2* ranges;
+  int64_t T;
+  uint32_t* class_list;   // [SORT_CLASSES][T]
+  uint32_t* class_count;  // [SORT_CLASSES]
+  uint32_t* order_count;  // [ORDER_BINS]
 };
+
+// Size classes of the per-tile bucket sorts (upper bounds, inclusive; longer
+// buckets go with the last class).
+constexpr int SORT_CLASSES = 6;
+constexpr int SORT_CLASS_BOUND[SORT_CLASSES] = {256, 2048, 4096, 6144, 8192, 12288};
+
+__device__ __forceinline__ int sort_class(uint32_t n) {
+  static_assert(SORT_CLASSES == 6, "one comparison per class bound");
+  constexpr uint32_t b0 = SORT_CLASS_BOUND[0], b1 = SORT_CLASS_BOUND[1], b2 = SORT_CLASS_BOUND[2],
+                     b3 = SORT_CLASS_BOUND[3], b4 = SORT_CLASS_BOUND[4];
+  return n == 0 ? -1
+                : (n <= b0 ? 0 : (n <= b1 ? 1 : (n <= b2 ? 2 : (n <= b3 ? 3 : (n <= b4 ? 4 : 5)))));
+}
+
+// Work-order bin of a list of n entries: floor(log2(n)) + 1, longest first.
+__device__ __forceinline__ int order_bin(uint32_t n) { return ORDER_BINS - 1 - (n ? 32 - __clz(n) : 0); }
+
+// Lanes of the warp that hold the same small value; `leader` is the first.
+__device__ __forceinline__ uint32_t same_value(int x, bool in, int& leader) {
+  const uint32_t m = __match_any_sync(0xffffffffu, in ? x : -1);
+  leader = __ffs(m) - 1;
+  return m;
+}
+
+// Appends every non-empty tile to its size class's list and counts the work
+// order's bins, a warp's tiles with one atomic per class and bin.  Runs ahead
+// of the scatter, over the whole grid (in the one-block scan these appends
+// were most of its time: 166 K tiles 260 us).
+__device__ void classify_tiles(const uint2* __restrict__ ranges, int64_t T, uint32_t* __restrict__ class_list,
+                               uint32_t* __restrict__ class_count, uint32_t* __restrict__ order_count) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < T; i0 += stride) {
+    const int64_t i = i0 + lane;
+    const uint2 r = i < T ? ranges[i] : make_uint2(0u, 0u);
+    const int cls = sort_class(r.y - r.x);
+    int lead;
+    const uint32_t mb = same_value(order_bin(r.y - r.x), i < T, lead);
+    if (i < T && lane == lead) atomicAdd(order_count + order_bin(r.y - r.x), (uint32_t)__popc(mb));
+    const uint32_t mc = same_value(cls, cls >= 0, lead);
+    uint32_t at = 0;
+    if (cls >= 0 && lane == lead) at = atomicAdd(class_count + cls, (uint32_t)__popc(mc));
+    at = __shfl_sync(0xffffffffu, at, lead);
+    if (cls >= 0) class_list[(size_t)cls * T + at + __popc(mc & lt_mask)] = (uint32_t)i;
+  }
+}
+
+// The work order of the persistent render kernels: tiles bucketed by
+// floor(log2(list length)), longest first.  Runs ahead of the first bucket sort.
+__device__ void order_tiles(const uint2* __restrict__ ranges, int64_t T, const uint32_t* __restrict__ order_count,
+                            uint32_t* __restrict__ order_cursor, uint32_t* __restrict__ order) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  static_assert(ORDER_BINS <= 64, "two bins per lane");
+  // each lane: the first position of bins 2 lane and 2 lane + 1
+  const uint32_t c0 = 2 * lane < ORDER_BINS ? order_count[2 * lane] : 0u,
+                 c1 = 2 * lane + 1 < ORDER_BINS ? order_count[2 * lane + 1] : 0u;
+  uint32_t x = c0 + c1;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  const uint32_t first0 = x - c0 - c1, first1 = x - c1;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < T; i0 += stride) {
+    const int64_t i = i0 + lane;
+    const uint2 r = i < T ? ranges[i] : make_uint2(0u, 0u);
+    const int b = order_bin(r.y - r.x);
+    int lead;
+    const uint32_t m = same_value(b, i < T, lead);
+    uint32_t at = 0;
+    if (i < T && lane == lead) at = atomicAdd(order_cursor + b, (uint32_t)__popc(m));
+    at = __shfl_sync(0xffffffffu, at, lead);
+    const uint32_t f0 = __shfl_sync(0xffffffffu, first0, b >> 1), f1 = __shfl_sync(0xffffffffu, first1, b >> 1);
+    if (i < T) order[((b & 1) ? f1 : f0) + at + __popc(m & lt_mask)] = (uint32_t)i;
+  }
+}
 
 // Visit every (record, tile) instance: the count pass adds them up per tile,
 // the scatter pass puts each record's composite (depth bits << 32 | surfel)
@@ -57,11 +142,15 @@ constexpr int BIN_KB = 4;
 
 template <bool SCATTER>
 __global__ void __launch_bounds__(256) k_tile_bin(const TileBinArgs A) {
+  chain_release();
+  chain_wait();
   if (SCATTER && A.hdr->status != 0) return;
+  if (SCATTER) classify_tiles(A.ranges, A.T, A.class_list, A.class_count, A.order_count);
   const int lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   // this thread's records only increase: follow the owning view forward
-  int v = find_view_by_record(A.views, A.V, min64((int64_t)blockIdx.x * blockDim.x + threadIdx.x, A.R - 1));
+  int v = A.R > 0 ? find_view_by_record(A.views, A.V, min64((int64_t)blockIdx.x * blockDim.x + threadIdx.x, A.R - 1))
+                  : 0;
   for (int64_t r0 = (int64_t)blockIdx.x * blockDim.x; r0 < A.R; r0 += stride) {
     const int64_t r = r0 + threadIdx.x;
     // 16 contiguous bytes per record (the records themselves are 80 bytes
@@ -126,87 +215,93 @@ __global__ void __launch_bounds__(256) k_tile_bin(const TileBinArgs A) {
   }
 }
 
-// Size classes of the per-tile bucket sorts (upper bounds, inclusive; longer
-// buckets go with the last class).
-constexpr int SORT_CLASSES = 6;
-constexpr int SORT_CLASS_BOUND[SORT_CLASSES] = {1024, 2048, 4096, 6144, 8192, 12288};
-
-__device__ __forceinline__ int sort_class(uint32_t n) {
-  static_assert(SORT_CLASSES == 6, "one comparison per class bound");
-  constexpr uint32_t b0 = SORT_CLASS_BOUND[0], b1 = SORT_CLASS_BOUND[1], b2 = SORT_CLASS_BOUND[2],
-                     b3 = SORT_CLASS_BOUND[3], b4 = SORT_CLASS_BOUND[4];
-  return n == 0 ? -1
-                : (n <= b0 ? 0 : (n <= b1 ? 1 : (n <= b2 ? 2 : (n <= b3 ? 3 : (n <= b4 ? 4 : 5)))));
-}
-
 // One block: exclusive scan of the tile counts -> ranges, scatter cursors,
-// total and the capacity check; every non-empty tile is appended to the list
-// of its sort size class.  Each thread takes SCAN_ITEMS consecutive tiles per
-// sweep, so a sweep covers 8192 tiles with one block-wide scan of the
-// threads' sums (a 64-view batch of about 770 K tiles takes 95 sweeps).
+// total and the capacity check.  Each thread takes SCAN_ITEMS consecutive
+// tiles per sweep, so a sweep covers 8192 tiles with one block-wide scan of
+// the threads' sums, the next sweep's counts already on their way.  The
+// counts are left zero for the next count pass, and the binning's small
+// counters (`small`) for the passes that follow.
 constexpr int SCAN_ITEMS = 8;
 
-__global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t* __restrict__ counts,
-                                                    uint32_t* __restrict__ cursors, uint2* __restrict__ ranges,
-                                                    int64_t T, Header* __restrict__ hdr, int64_t cap,
-                                                    uint32_t* __restrict__ class_list,
-                                                    uint32_t* __restrict__ class_count) {
+__global__ void __launch_bounds__(1024) k_tile_scan(uint32_t* __restrict__ counts, uint32_t* __restrict__ cursors,
+                                                    uint2* __restrict__ ranges, int64_t T, Header* __restrict__ hdr,
+                                                    int64_t cap, uint32_t* __restrict__ small, int n_small) {
   __shared__ unsigned long long s_w[32];
   __shared__ unsigned long long s_carry;
+  chain_release();
+  chain_wait();
   if (threadIdx.x == 0) s_carry = 0;
-  __syncthreads();
+  for (int i = threadIdx.x; i < n_small; i += 1024) small[i] = 0u;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const uint32_t lt_mask = (1u << lane) - 1u;
+  uint32_t next[SCAN_ITEMS];
+  // (the arrays are 256-byte aligned and a thread's tiles start at a multiple of 8)
+  auto load = [&](int64_t i0) {
+    if (i0 + SCAN_ITEMS <= T) {
+      const uint4 a = *reinterpret_cast<const uint4*>(counts + i0), b = *reinterpret_cast<const uint4*>(counts + i0 + 4);
+      next[0] = a.x; next[1] = a.y; next[2] = a.z; next[3] = a.w;
+      next[4] = b.x; next[5] = b.y; next[6] = b.z; next[7] = b.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < SCAN_ITEMS; j++) next[j] = i0 + j < T ? counts[i0 + j] : 0u;
+    }
+  };
+  load((int64_t)threadIdx.x * SCAN_ITEMS);
+  __syncthreads();
   for (int64_t base = 0; base < T; base += 1024 * SCAN_ITEMS) {
     const int64_t i0 = base + (int64_t)threadIdx.x * SCAN_ITEMS;
     uint32_t v[SCAN_ITEMS];
     unsigned long long sum = 0;
 #pragma unroll
     for (int j = 0; j < SCAN_ITEMS; j++) {
-      v[j] = i0 + j < T ? counts[i0 + j] : 0u;
+      v[j] = next[j];
       sum += v[j];
     }
+    load(i0 + 1024 * SCAN_ITEMS);
     unsigned long long x = sum;
+#pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
       if (lane >= o) x += y;
     }
     if (lane == 31) s_w[wid] = x;
     __syncthreads();
-    if (wid == 0) {
-      unsigned long long w = s_w[lane];
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xffffffffu, w, o);
-        if (lane >= o) w += y;
-      }
-      s_w[lane] = w;
+    // every warp scans the warps' sums
+    unsigned long long w = s_w[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += y;
     }
-    __syncthreads();
-    unsigned long long incl = x - sum + (wid > 0 ? s_w[wid - 1] : 0ull) + s_carry;
+    const unsigned long long carry = s_carry, total = __shfl_sync(0xffffffffu, w, 31);
+    const unsigned long long before = __shfl_sync(0xffffffffu, w, wid > 0 ? wid - 1 : 0);
+    unsigned long long incl = carry + (wid > 0 ? before : 0ull) + x - sum;
+    uint2 rg[SCAN_ITEMS];
 #pragma unroll
     for (int j = 0; j < SCAN_ITEMS; j++) {
-      const int64_t i = i0 + j;
       const unsigned long long start = incl;
       incl += v[j];
-      const bool fits = incl <= (unsigned long long)cap;
-      if (i < T) {
-        ranges[i] = fits ? make_uint2((uint32_t)start, (uint32_t)incl) : make_uint2(0u, 0u);
-        cursors[i] = fits ? (uint32_t)start : 0u;
-      }
-      // append the tile to its size class's list (order within a list is free)
-      const int cls = (i < T && fits) ? sort_class(v[j]) : -1;
+      rg[j] = incl <= (unsigned long long)cap ? make_uint2((uint32_t)start, (uint32_t)incl) : make_uint2(0u, 0u);
+    }
+    if (i0 + SCAN_ITEMS <= T) {
 #pragma unroll
-      for (int c = 0; c < SORT_CLASSES; c++) {
-        const uint32_t m = __ballot_sync(0xffffffffu, cls == c);
-        if (!m) continue;
-        uint32_t at = 0;
-        if (lane == 0) at = atomicAdd(&class_count[c], (uint32_t)__popc(m));
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if (cls == c) class_list[(size_t)c * T + at + __popc(m & lt_mask)] = (uint32_t)i;
+      for (int j = 0; j < SCAN_ITEMS; j += 2)
+        *reinterpret_cast<uint4*>(ranges + i0 + j) = make_uint4(rg[j].x, rg[j].y, rg[j + 1].x, rg[j + 1].y);
+#pragma unroll
+      for (int j = 0; j < SCAN_ITEMS; j += 4) {
+        *reinterpret_cast<uint4*>(cursors + i0 + j) = make_uint4(rg[j].x, rg[j + 1].x, rg[j + 2].x, rg[j + 3].x);
+        *reinterpret_cast<uint4*>(counts + i0 + j) = make_uint4(0u, 0u, 0u, 0u);
       }
+    } else {
+#pragma unroll
+      for (int j = 0; j < SCAN_ITEMS; j++)
+        if (i0 + j < T) {
+          ranges[i0 + j] = rg[j];
+          cursors[i0 + j] = rg[j].x;
+          counts[i0 + j] = 0u;
+        }
     }
     __syncthreads();
-    if (threadIdx.x == 1023) s_carry = incl;
+    if (threadIdx.x == 0) s_carry = carry + total;
     __syncthreads();
   }
   if (threadIdx.x == 0) {
@@ -565,7 +660,7 @@ __device__ void sort_bucket_reg(const unsigned long long* __restrict__ g, int n,
   __syncthreads();
   uint32_t dmn = 0xffffffffu, dmx = 0u, imn = 0xffffffffu, imx = 0u;
   for (int i = threadIdx.x; i < n; i += NT) {
-    const unsigned long long x = g[i];
+    const unsigned long long x = __ldcg(g + i);
     sa[i] = x;
     const uint32_t d = (uint32_t)(x >> 32), s = (uint32_t)x;
     dmn = min(dmn, d); dmx = max(dmx, d); imn = min(imn, s); imx = max(imx, s);
@@ -624,10 +719,10 @@ __device__ void sort_bucket_reg(const unsigned long long* __restrict__ g, int n,
   }
 }
 
-// Per-tile bucket sorts in three size classes, each a persistent launch over
-// its class's tile list with shared memory sized for the class (so short
-// buckets run several CTAs per SM); the last class also takes the buckets
-// longer than its capacity and sorts those in global memory.
+// Per-tile bucket sorts in size classes, each a persistent launch over its
+// class's tile list with shared memory sized for the class (so short buckets
+// run several CTAs per SM); the last class also takes the buckets longer than
+// its capacity and sorts those in global memory.
 struct SegArgs {
   const uint2* ranges;
   unsigned long long* bucket;   // scattered composites (sorted in place for the oversized buckets)
@@ -639,7 +734,211 @@ struct SegArgs {
   const uint32_t* list;         // this class's tiles
   const uint32_t* list_count;   // their number
   uint32_t* queue;              // this class's work counter
+  // first class: the work order of the render kernels
+  int64_t T;
+  const uint32_t* order_count;
+  uint32_t* order_cursor;
+  uint32_t* order;
 };
+
+// Short buckets (at most 32 * WS_ITEMS composites): one warp each, no block
+// barriers (six CTAs per SM; at 9 warps per SM, without the register bound,
+// latency-bound: 269 against 201 us for one keyframe x 8 views, preprocess and
+// binning).  The same two radix passes as sort_bucket_reg: the keys go from
+// global memory to registers, the first pass ranks them by shared atomics, the
+// second (stable) by ballot multisplit against one counter per digit, each
+// scan of the 256 counters taking 8 per lane.  Runs of ties are ranked in
+// parallel as the bucket is written out; a run longer than 64 takes stable
+// passes over the whole relative composite instead.  A 256-thread CTA per
+// bucket spent most of a short one at its barriers: buckets of about 150
+// entries (12 uneven submaps, 166 K tiles) 785 us.
+constexpr int WS_ITEMS = 8;
+constexpr int WS_WARPS = 4;  // buckets (warps) per CTA; they share nothing
+struct WarpSortSmem {
+  unsigned long long key[32 * WS_ITEMS];
+  uint32_t cnt[256];
+};
+
+__device__ __forceinline__ void warp_scan256(uint32_t* cnt, int lane) {
+  uint4 a = reinterpret_cast<uint4*>(cnt)[2 * lane], b = reinterpret_cast<uint4*>(cnt)[2 * lane + 1];
+  const uint32_t sum = a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w;
+  uint32_t x = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  uint32_t run = x - sum, t;
+  t = a.x; a.x = run; run += t;
+  t = a.y; a.y = run; run += t;
+  t = a.z; a.z = run; run += t;
+  t = a.w; a.w = run; run += t;
+  t = b.x; b.x = run; run += t;
+  t = b.y; b.y = run; run += t;
+  t = b.z; b.z = run; run += t;
+  b.w = run;
+  reinterpret_cast<uint4*>(cnt)[2 * lane] = a;
+  reinterpret_cast<uint4*>(cnt)[2 * lane + 1] = b;
+  __syncwarp();
+}
+
+__device__ __forceinline__ void warp_clear256(uint32_t* cnt, int lane) {
+  reinterpret_cast<uint4*>(cnt)[2 * lane] = make_uint4(0u, 0u, 0u, 0u);
+  reinterpret_cast<uint4*>(cnt)[2 * lane + 1] = make_uint4(0u, 0u, 0u, 0u);
+  __syncwarp();
+}
+
+// One stable pass by the digit (composite's sort key >> shift) & 255 over S.key.
+template <typename KeyOf>
+__device__ __forceinline__ void warp_pass_stable(WarpSortSmem& S, int n, int shift, int lane, const KeyOf& key_of) {
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  const int nr = (n + 31) >> 5;
+  unsigned long long key[WS_ITEMS];
+  uint32_t off[WS_ITEMS];
+  warp_clear256(S.cnt, lane);
+#pragma unroll
+  for (int k = 0; k < WS_ITEMS; k++) {
+    if (k >= nr) break;
+    const bool valid = k * 32 + lane < n;
+    key[k] = valid ? S.key[k * 32 + lane] : 0ull;
+    const uint32_t d = valid ? (uint32_t)(key_of(key[k]) >> shift) & 0xffu : 0u;
+    uint32_t peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+    for (int bit = 0; bit < 8; bit++) {
+      const bool on = (d >> bit) & 1u;
+      const uint32_t bal = __ballot_sync(0xffffffffu, on);
+      peers &= on ? bal : ~bal;
+    }
+    const int leader = __ffs(peers) - 1;
+    uint32_t pre = 0;
+    if (valid && lane == leader) {
+      pre = S.cnt[d];
+      S.cnt[d] = pre + __popc(peers);
+    }
+    pre = __shfl_sync(0xffffffffu, pre, leader & 31);
+    off[k] = (d << 16) | (pre + __popc(peers & lt_mask));
+    __syncwarp();
+  }
+  warp_scan256(S.cnt, lane);
+#pragma unroll
+  for (int k = 0; k < WS_ITEMS; k++)
+    if (k < nr && k * 32 + lane < n) S.key[S.cnt[off[k] >> 16] + (off[k] & 0xffffu)] = key[k];
+  __syncwarp();
+}
+
+__device__ void warp_sort_bucket(const unsigned long long* __restrict__ g, int n, WarpSortSmem& S, int lane,
+                                 uint64_t tile, uint64_t* __restrict__ okeys, uint32_t* __restrict__ ovals) {
+  const int nr = (n + 31) >> 5;
+  uint32_t dmin, dbits;
+  int lsb;
+  {
+    unsigned long long key[WS_ITEMS];
+    uint32_t dmn = 0xffffffffu, dmx = 0u;
+#pragma unroll
+    for (int k = 0; k < WS_ITEMS; k++)
+      if (k < nr) key[k] = k * 32 + lane < n ? __ldg(g + k * 32 + lane) : 0ull;
+    warp_clear256(S.cnt, lane);
+#pragma unroll
+    for (int k = 0; k < WS_ITEMS; k++)
+      if (k < nr && k * 32 + lane < n) {
+        const uint32_t d = (uint32_t)(key[k] >> 32);
+        dmn = min(dmn, d);
+        dmx = max(dmx, d);
+      }
+    dmin = __reduce_min_sync(0xffffffffu, dmn);
+    dbits = (uint32_t)bits_of(__reduce_max_sync(0xffffffffu, dmx) - dmin);
+    lsb = max((int)dbits - 16, 0);
+    // first pass (the order of equal digits is free)
+    uint32_t off[WS_ITEMS];
+#pragma unroll
+    for (int k = 0; k < WS_ITEMS; k++)
+      if (k < nr && k * 32 + lane < n) {
+        const uint32_t d = (((uint32_t)(key[k] >> 32) - dmin) >> lsb) & 0xffu;
+        off[k] = (d << 16) | atomicAdd(&S.cnt[d], 1u);
+      }
+    __syncwarp();
+    warp_scan256(S.cnt, lane);
+#pragma unroll
+    for (int k = 0; k < WS_ITEMS; k++)
+      if (k < nr && k * 32 + lane < n) S.key[S.cnt[off[k] >> 16] + (off[k] & 0xffffu)] = key[k];
+    __syncwarp();
+  }
+  if ((int)dbits - lsb > 8)
+    warp_pass_stable(S, n, 8, lane, [&](unsigned long long x) { return ((uint32_t)(x >> 32) - dmin) >> lsb; });
+  auto top = [&](unsigned long long x) -> uint32_t { return ((uint32_t)(x >> 32) - dmin) >> lsb; };
+  auto emit = [&](int p, unsigned long long key) {
+    okeys[p] = tile | (key >> 32);
+    ovals[p] = (uint32_t)key;
+  };
+  bool long_run = false;
+  for (int i0 = 0; i0 < n; i0 += 32) {
+    const int i = i0 + lane;
+    const bool in = i < n;
+    const unsigned long long key = in ? S.key[i] : 0ull;
+    const uint32_t d = top(key);
+    // the neighbours' top bits: the adjacent lanes' entries, across rounds a load
+    uint32_t dp = __shfl_up_sync(0xffffffffu, d, 1), dn = __shfl_down_sync(0xffffffffu, d, 1);
+    if (lane == 0 && in && i > 0) dp = top(S.key[i - 1]);
+    if (lane == 31 && i + 1 < n) dn = top(S.key[i + 1]);
+    if (!in) continue;
+    if (!((i > 0 && dp == d) || (i + 1 < n && dn == d))) {
+      emit(i, key);
+      continue;
+    }
+    int s = i, e = i;
+    while (s > 0 && i - s < 64 && top(S.key[s - 1]) == d) s--;
+    while (e + 1 < n && e - i < 64 && top(S.key[e + 1]) == d) e++;
+    if (e - s >= 64) {
+      long_run = true;
+      continue;
+    }
+    int rank = 0;
+    for (int y = s; y <= e; y++) rank += S.key[y] < key ? 1 : 0;
+    emit(s + rank, key);
+  }
+  if (__any_sync(0xffffffffu, long_run)) {
+    uint32_t imn = 0xffffffffu, imx = 0u;
+    for (int i = lane; i < n; i += 32) {
+      imn = min(imn, (uint32_t)S.key[i]);
+      imx = max(imx, (uint32_t)S.key[i]);
+    }
+    const uint32_t imin = __reduce_min_sync(0xffffffffu, imn);
+    const int ibits = bits_of(__reduce_max_sync(0xffffffffu, imx) - imin);
+    for (int shift = 0; shift < (int)dbits + ibits; shift += 8)
+      warp_pass_stable(S, n, shift, lane, [&](unsigned long long x) {
+        return (unsigned long long)((uint32_t)(x >> 32) - dmin) << ibits | (unsigned long long)((uint32_t)x - imin);
+      });
+    for (int i = lane; i < n; i += 32) emit(i, S.key[i]);
+  }
+}
+
+__global__ void __launch_bounds__(WS_WARPS * 32, 6) k_tile_sort_warp(const SegArgs A) {
+  __shared__ __align__(16) WarpSortSmem s_sort[WS_WARPS];
+  chain_wait();
+  chain_release();  // after the wait: the next class starts without one (see k_tile_sort)
+  if (A.hdr->status != 0) return;
+  order_tiles(A.ranges, A.T, A.order_count, A.order_cursor, A.order);
+  const int lane = threadIdx.x & 31;
+  WarpSortSmem& S = s_sort[threadIdx.x >> 5];
+  const uint32_t n_tiles = *A.list_count;
+  // buckets of one class are alike, so the warps take them in turn, and know
+  // the next one's place while they sort this one
+  const uint32_t step = gridDim.x * WS_WARPS;
+  uint32_t q = blockIdx.x * WS_WARPS + (threadIdx.x >> 5);
+  uint32_t t_next = q < n_tiles ? A.list[q] : 0u;
+  uint2 r_next = q < n_tiles ? A.ranges[t_next] : make_uint2(0u, 0u);
+  for (; q < n_tiles; q += step) {
+    const uint32_t t = t_next;
+    const uint2 rg = r_next;
+    if (q + step < n_tiles) {
+      t_next = A.list[q + step];
+      r_next = A.ranges[t_next];
+    }
+    if (!s2d_check(rg.x <= rg.y && (int64_t)rg.y <= A.cap && rg.y - rg.x <= 32 * WS_ITEMS, A.hdr)) continue;
+    warp_sort_bucket(A.bucket + rg.x, (int)(rg.y - rg.x), S, lane, (uint64_t)t << 32, A.keys + rg.x, A.vals + rg.x);
+    __syncwarp();
+  }
+}
 
 template <int NWARPS, int ITEMS>
 struct SegClass {
@@ -657,11 +956,10 @@ template <int NWARPS, int ITEMS, bool LAST>
 // (binning 10.01 -> 9.82 ms for the first class, 9.82 -> 9.62 ms for the
 // second, on the 32-keyframe submap; sorting the 6145..8192 buckets there
 // instead of in the 1024-thread class at one CTA per SM: 9.63 -> 9.37 ms, and
-// 9.46 ms at 2 CTAs per SM without the spills).  The <= 1024 and 1025..2048
-// classes (256 threads, 13 and 21 KB) run 6 CTAs per SM, which matters where
-// buckets are short (64 uneven submaps: binning 13.38 -> 11.37 ms for the
-// first, and 11.62 -> 11.35 ms for taking the 1025..2048 buckets out of the
-// 512-thread class).
+// 9.46 ms at 2 CTAs per SM without the spills).  The 257..2048 class (256
+// threads, 21 KB) runs 6 CTAs per SM, which matters where buckets are short
+// (64 uneven submaps: binning 11.62 -> 11.35 ms for taking the 1025..2048
+// buckets out of the 512-thread class).
 __global__ void __launch_bounds__(NWARPS * 32, NWARPS == 16 ? 3 : (NWARPS == 8 ? 6 : 1)) k_tile_sort(const SegArgs A) {
   using C = SegClass<NWARPS, ITEMS>;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -674,16 +972,21 @@ __global__ void __launch_bounds__(NWARPS * 32, NWARPS == 16 ? 3 : (NWARPS == 8 ?
                                               ((RegSortSmem<NWARPS>::CNT_BYTES + 15) & ~(size_t)15));
   uint32_t* red = tot + 32;
   __shared__ uint32_t s_q;
-  if (A.hdr->status != 0) return;
-  const uint32_t n_tiles = *A.list_count;
+  // The classes sort disjoint buckets, so a class runs beside the one before
+  // it (8 keyframes x 8 views: 1215 -> 1150 us for preprocess and binning):
+  // the scatter pass they depend on was complete before the first class let
+  // them start, and the wait for the class before comes last.  Until then
+  // what the scatter wrote is read through L2.
+  chain_release();
+  const uint32_t n_tiles = __ldcg(&A.hdr->status) != 0 ? 0u : __ldcg(A.list_count);
   for (;;) {
     if (threadIdx.x == 0) s_q = atomicAdd(A.queue, 1u);
     __syncthreads();
     const uint32_t q = s_q;
     __syncthreads();
     if (q >= n_tiles) break;
-    const uint32_t t = A.list[q];
-    const uint2 rg = A.ranges[t];
+    const uint32_t t = __ldcg(A.list + q);
+    const uint2 rg = __ldcg(A.ranges + t);
     if (!s2d_check(rg.x <= rg.y && (int64_t)rg.y <= A.cap, A.hdr)) continue;
     const int n = (int)(rg.y - rg.x);
     const uint64_t tile = (uint64_t)t << 32;
@@ -691,6 +994,7 @@ __global__ void __launch_bounds__(NWARPS * 32, NWARPS == 16 ? 3 : (NWARPS == 8 ?
       sort_bucket_reg<NWARPS, ITEMS>(A.bucket + rg.x, n, sa, sb, cnt, tot, red, tile, A.keys + rg.x, A.vals + rg.x);
     } else {
       uint32_t* c32 = reinterpret_cast<uint32_t*>(smem);
+      chain_wait();
       sort_bucket_any<NWARPS>(A.bucket + rg.x, A.scratch + rg.x, n, c32, c32 + (NWARPS + 1) * 256);
       const unsigned long long* res = A.bucket + rg.x;
       for (int i = threadIdx.x; i < n; i += NWARPS * 32) {
@@ -701,6 +1005,7 @@ __global__ void __launch_bounds__(NWARPS * 32, NWARPS == 16 ? 3 : (NWARPS == 8 ?
     }
     __syncthreads();
   }
+  chain_wait();
 }
 
 template <int NWARPS, int ITEMS, bool LAST>
@@ -713,19 +1018,26 @@ static cudaError_t launch_tile_sort_class(const SegArgs& S, cudaStream_t st) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, C::THREADS, C::SMEM);
     if (per_sm < 1) per_sm = 1;
   }
-  k<<<per_sm * sm_count(), C::THREADS, C::SMEM, st>>>(S);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_chained(k, per_sm * sm_count(), C::THREADS, C::SMEM, st, S);
 }
 
+// Count, scan, scatter (which also lists the tiles by size class) and the
+// classes' sorts (the first of which also writes the work order), each chained
+// to the one before.  With separate passes for the order, a launch per class
+// whatever the range sizes, memsets in between and unchained launches: one
+// 128x96 view 85 -> 45 us, one 512x384 view of its keyframe 109 -> 69, 8 views
+// of it 277 -> 156, 12 uneven submaps 1425 -> 745, 24 keyframes x 24 views
+// 6220 -> 5870.
 cudaError_t launch_bin_tiles(const Layout& L, const RastParams& P, char* ws, cudaStream_t st) {
-  if (L.R <= 0 || L.T <= 0) return cudaSuccess;
+  if (L.T <= 0) return cudaSuccess;
   Header* hdr = reinterpret_cast<Header*>(ws + L.header);
   uint32_t* counts = reinterpret_cast<uint32_t*>(ws + L.tile_count);
   uint32_t* cursors = reinterpret_cast<uint32_t*>(ws + L.tile_cursor);
   uint2* ranges = reinterpret_cast<uint2*>(ws + L.ranges);
-  cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(uint32_t) * (size_t)L.T, st);
-  if (e != cudaSuccess) return e;
+  // small counters: work-order bins and cursors, per class its queue and list size
+  uint32_t* small = reinterpret_cast<uint32_t*>(ws + L.tile_hist);
+  uint32_t *order_count = small, *order_cursor = small + ORDER_BINS, *queues = small + 2 * ORDER_BINS;
+  static_assert(2 * ORDER_BINS + 2 * SORT_CLASSES <= TILE_HIST_WORDS, "the small counters fit");
   TileBinArgs A;
   A.bins = reinterpret_cast<const uint4*>(ws + L.bins);
   A.views = reinterpret_cast<const DView*>(ws + L.views);
@@ -737,19 +1049,24 @@ cudaError_t launch_bin_tiles(const Layout& L, const RastParams& P, char* ws, cud
   A.bucket = reinterpret_cast<unsigned long long*>(ws + L.keys1);
   A.cap = L.cap;
   A.hdr = hdr;
-  const int64_t blocks = (L.R + 255) / 256;
-  const int grid0 = (int)min64(blocks, (int64_t)sm_count() * 16), grid1 = grid0;
-  k_tile_bin<false><<<grid0, 256, 0, st>>>(A);
-  count_launches(1);
-  uint32_t* queues = reinterpret_cast<uint32_t*>(ws + L.tile_hist) + ORDER_BINS;  // per class: queue, list size
-  uint32_t* class_list = reinterpret_cast<uint32_t*>(ws + L.tile_class);
-  e = cudaMemsetAsync(queues, 0, 2 * SORT_CLASSES * sizeof(uint32_t), st);
+  A.ranges = ranges;
+  A.T = L.T;
+  A.class_list = reinterpret_cast<uint32_t*>(ws + L.tile_class);
+  A.class_count = queues + SORT_CLASSES;
+  A.order_count = order_count;
+  const int64_t work = L.R > L.T ? L.R : L.T;
+  const int grid = (int)min64((work + 255) / 256, (int64_t)sm_count() * 16);
+  cudaError_t e = cudaSuccess;
+  // the counts are zero: cleared by the preprocess, and again by each scan
+  if (L.R > 0) {
+    e = launch_chained(k_tile_bin<false>, grid, 256, 0, st, A);
+    if (e != cudaSuccess) return e;
+  }
+  e = launch_chained(k_tile_scan, 1, 1024, 0, st, counts, cursors, ranges, L.T, hdr, L.cap, small, TILE_HIST_WORDS);
   if (e != cudaSuccess) return e;
-  k_tile_scan<<<1, 1024, 0, st>>>(counts, cursors, ranges, L.T, hdr, L.cap, class_list, queues + SORT_CLASSES);
-  count_launches(1);
   A.counts = cursors;
-  k_tile_bin<true><<<grid1, 256, 0, st>>>(A);
-  count_launches(1);
+  e = launch_chained(k_tile_bin<true>, grid, 256, 0, st, A);
+  if (e != cudaSuccess) return e;
   SegArgs S;
   S.ranges = ranges;
   S.bucket = A.bucket;
@@ -758,16 +1075,31 @@ cudaError_t launch_bin_tiles(const Layout& L, const RastParams& P, char* ws, cud
   S.vals = reinterpret_cast<uint32_t*>(ws + L.vals0);
   S.hdr = hdr;
   S.cap = L.cap;
-  static_assert(SegClass<8, 4>::CAP == SORT_CLASS_BOUND[0] && SegClass<8, 8>::CAP == SORT_CLASS_BOUND[1] &&
+  S.T = L.T;
+  S.order_count = order_count;
+  S.order_cursor = order_cursor;
+  S.order = reinterpret_cast<uint32_t*>(ws + L.tile_order);
+  static_assert(32 * WS_ITEMS == SORT_CLASS_BOUND[0] && SegClass<8, 8>::CAP == SORT_CLASS_BOUND[1] &&
                     SegClass<16, 8>::CAP == SORT_CLASS_BOUND[2] && SegClass<16, 12>::CAP == SORT_CLASS_BOUND[3] &&
                     SegClass<16, 16>::CAP == SORT_CLASS_BOUND[4] && SegClass<32, 12>::CAP == SORT_CLASS_BOUND[5],
                 "class capacities match the class bounds");
   for (int c = 0; c < SORT_CLASSES; c++) {
-    S.list = class_list + (size_t)c * L.T;
-    S.list_count = queues + SORT_CLASSES + c;
+    // a surfel has one entry per tile, so no bucket is longer than a view's surfel range
+    if (c > 0 && L.max_range <= SORT_CLASS_BOUND[c - 1]) break;
+    S.list = A.class_list + (size_t)c * L.T;
+    S.list_count = A.class_count + c;
     S.queue = queues + c;
     switch (c) {
-      case 0: e = launch_tile_sort_class<8, 4, false>(S, st); break;
+      case 0: {
+        static int per_sm = -1;
+        if (per_sm < 0) {
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_sort_warp, WS_WARPS * 32, 0);
+          if (per_sm < 1) per_sm = 1;
+        }
+        const int64_t most = (L.T + WS_WARPS - 1) / WS_WARPS;
+        e = launch_chained(k_tile_sort_warp, (int)min64(most, (int64_t)per_sm * sm_count()), WS_WARPS * 32, 0, st, S);
+        break;
+      }
       case 1: e = launch_tile_sort_class<8, 8, false>(S, st); break;
       case 2: e = launch_tile_sort_class<16, 8, false>(S, st); break;
       case 3: e = launch_tile_sort_class<16, 12, false>(S, st); break;
@@ -941,64 +1273,6 @@ cudaError_t launch_sort(uint64_t* keys0, uint32_t* vals0, uint64_t* keys1, uint3
     cur ^= 1;
   }
   *final_buffer = cur;
-  return cudaGetLastError();
-}
-
-// Work order for the persistent render kernels: tiles bucketed by
-// floor(log2(list length)), longest first (a counting sort on the bucket).
-__global__ void __launch_bounds__(256) k_order_hist(const uint2* __restrict__ ranges, int64_t T,
-                                                    uint32_t* __restrict__ bins) {
-  __shared__ uint32_t s_b[ORDER_BINS];
-  for (int i = threadIdx.x; i < ORDER_BINS; i += blockDim.x) s_b[i] = 0;
-  __syncthreads();
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < T; t += (int64_t)gridDim.x * blockDim.x) {
-    const uint2 r = ranges[t];
-    const uint32_t len = r.y - r.x;
-    const int b = len ? 32 - __clz(len) : 0;  // 0..32, larger = longer
-    atomicAdd(&s_b[ORDER_BINS - 1 - b], 1u);
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < ORDER_BINS; i += blockDim.x)
-    if (s_b[i]) atomicAdd(&bins[i], s_b[i]);
-}
-
-__global__ void k_order_scan(uint32_t* __restrict__ bins) {
-  if (threadIdx.x == 0) {
-    uint32_t acc = 0;
-    for (int i = 0; i < ORDER_BINS; i++) {
-      uint32_t c = bins[i];
-      bins[i] = acc;
-      acc += c;
-    }
-  }
-}
-
-__global__ void __launch_bounds__(256) k_order_scatter(const uint2* __restrict__ ranges, int64_t T,
-                                                       uint32_t* __restrict__ bins, uint32_t* __restrict__ order) {
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < T; t += (int64_t)gridDim.x * blockDim.x) {
-    const uint2 r = ranges[t];
-    const uint32_t len = r.y - r.x;
-    const int b = len ? 32 - __clz(len) : 0;
-    const uint32_t pos = atomicAdd(&bins[ORDER_BINS - 1 - b], 1u);
-    order[pos] = (uint32_t)t;
-  }
-}
-
-cudaError_t launch_order(const Layout& L, char* ws, cudaStream_t st) {
-  if (L.T <= 0) return cudaSuccess;
-  const uint2* ranges = reinterpret_cast<const uint2*>(ws + L.ranges);
-  uint32_t* bins = reinterpret_cast<uint32_t*>(ws + L.tile_hist);
-  uint32_t* order = reinterpret_cast<uint32_t*>(ws + L.tile_order);
-  cudaError_t e = cudaMemsetAsync(bins, 0, sizeof(uint32_t) * ORDER_BINS, st);
-  if (e != cudaSuccess) return e;
-  int g2 = (int)min64((L.T + 255) / 256, (int64_t)sm_count() * 4);
-  if (g2 < 1) g2 = 1;
-  k_order_hist<<<g2, 256, 0, st>>>(ranges, L.T, bins);
-  count_launches(1);
-  k_order_scan<<<1, 32, 0, st>>>(bins);
-  count_launches(1);
-  k_order_scatter<<<g2, 256, 0, st>>>(ranges, L.T, bins, order);
-  count_launches(1);
   return cudaGetLastError();
 }
 

@@ -22,31 +22,51 @@
 namespace s2d {
 
 // ---------------------------------------------------------------------------
-// Table upload: copies a small host table into the workspace through the
-// kernel's parameter space (no host memory is touched at run time, so the
-// call can be captured in a CUDA graph).
+// Setup: the header and the tables (contiguous at the start of the workspace)
+// through the kernel's parameter space, so that no host memory is touched at
+// run time and the call can be captured in a CUDA graph, and zero tile counts
+// for the binning.  The parameter block comes in three sizes: a large one
+// costs the host more per launch.
 // ---------------------------------------------------------------------------
-constexpr int kUploadBytes = 16384;
+template <int BYTES>
 struct UploadBlob {
-  uint4 data[kUploadBytes / 16];
+  uint4 data[BYTES / 16];
 };
 
-__global__ void k_upload(const UploadBlob blob, uint4* __restrict__ dst, int n16) {
-  for (int i = threadIdx.x; i < n16; i += blockDim.x) dst[i] = blob.data[i];
+template <int BYTES>
+__global__ void __launch_bounds__(256) k_setup(const UploadBlob<BYTES> blob, uint4* __restrict__ dst, int n16,
+                                               uint32_t* __restrict__ zero, int64_t n_zero) {
+  chain_release();
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < n16; i += 256) dst[i] = blob.data[i];
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n_zero; i += (int64_t)gridDim.x * 256) zero[i] = 0u;
 }
 
-cudaError_t launch_upload(const void* host_src, size_t bytes, void* dst, cudaStream_t st) {
-  const char* src = static_cast<const char*>(host_src);
-  UploadBlob blob;
-  for (size_t off = 0; off < bytes; off += kUploadBytes) {
-    size_t n = bytes - off < (size_t)kUploadBytes ? bytes - off : (size_t)kUploadBytes;
-    size_t n16 = (n + 15) / 16;
-    memset(&blob, 0, sizeof(blob));
-    memcpy(&blob, src + off, n);
-    k_upload<<<1, 256, 0, st>>>(blob, reinterpret_cast<uint4*>(static_cast<char*>(dst) + off), (int)n16);
-    count_launches(1);
-    cudaError_t e = cudaGetLastError();
+template <int BYTES>
+static cudaError_t run_setup(const char* src, size_t n, char* dst, uint32_t* zero, int64_t n_zero, cudaStream_t st) {
+  UploadBlob<BYTES> blob;
+  memcpy(&blob, src, n);
+  memset(reinterpret_cast<char*>(&blob) + n, 0, sizeof(blob) - n);
+  const int grid = (int)max64(1, min64((n_zero + 2047) / 2048, (int64_t)sm_count() * 4));
+  k_setup<BYTES><<<grid, 256, 0, st>>>(blob, reinterpret_cast<uint4*>(dst), (int)((n + 15) / 16), zero, n_zero);
+  count_launches(1);
+  return cudaGetLastError();
+}
+
+// Writes `bytes` of tables at the workspace's start and clears the tile counts.
+cudaError_t launch_setup(const void* tables, size_t bytes, const Layout& L, char* ws, cudaStream_t st) {
+  constexpr size_t kLargest = 16384;
+  const char* src = static_cast<const char*>(tables);
+  uint32_t* zero = reinterpret_cast<uint32_t*>(ws + L.tile_count);
+  int64_t n_zero = L.T;
+  for (size_t off = 0; off < bytes; off += kLargest) {
+    const size_t n = bytes - off < kLargest ? bytes - off : kLargest;
+    char* dst = ws + L.header + off;
+    cudaError_t e = n <= 1024   ? run_setup<1024>(src + off, n, dst, zero, n_zero, st)
+                    : n <= 4096 ? run_setup<4096>(src + off, n, dst, zero, n_zero, st)
+                                : run_setup<(int)kLargest>(src + off, n, dst, zero, n_zero, st);
     if (e != cudaSuccess) return e;
+    n_zero = 0;
   }
   return cudaSuccess;
 }
@@ -249,6 +269,8 @@ __device__ __forceinline__ uint32_t project_one(const PreArgs& A, const DView& v
 }
 
 __global__ void __launch_bounds__(256, 3) k_preprocess(const PreArgs A) {
+  chain_release();
+  chain_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   unsigned long long vis = 0;
   for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < A.n_work; w += stride) {
@@ -304,9 +326,7 @@ cudaError_t launch_preprocess(const splat2d_surfels* S, const Layout& L, const R
   int64_t blocks = (n_work + 255) / 256;
   int64_t cap = (int64_t)sm_count() * 16;
   if (blocks > cap) blocks = cap;
-  k_preprocess<<<(unsigned)blocks, 256, 0, st>>>(A);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_chained(k_preprocess, (int)blocks, 256, 0, st, A);
 }
 
 // ---------------------------------------------------------------------------
@@ -332,6 +352,8 @@ constexpr int kPoseSlots = 64;  // per-block pose accumulators (views)
 __global__ void __launch_bounds__(256, 4) k_preprocess_bwd(const PreBwdArgs A) {
   __shared__ float s_pose[kPoseSlots][6];
   __shared__ int s_vfirst;
+  chain_release();
+  chain_wait();
   // a failed binning (instance capacity exceeded): nothing was accumulated
   if (A.hdr->status != 0) return;
   const int64_t wlo = (int64_t)blockIdx.x * A.per_block;
@@ -544,9 +566,7 @@ cudaError_t launch_preprocess_bwd(const splat2d_surfels* S, const Layout& L, con
   if (per < 256) per = 256;
   A.per_block = per;
   int64_t blocks = (n_work + per - 1) / per;
-  k_preprocess_bwd<<<(unsigned)blocks, 256, 0, st>>>(A);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_chained(k_preprocess_bwd, (int)blocks, 256, 0, st, A);
 }
 
 }  // namespace s2d

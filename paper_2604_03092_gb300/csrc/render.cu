@@ -402,6 +402,8 @@ __global__ void __launch_bounds__(TW* TH, 3) k_render_fwd(const RenderArgs A) {
   const uint32_t lt_mask = (1u << lane) - 1u;
   const RastParams& P = A.P;
   uint32_t n_eval = 0, n_blend = 0;
+  chain_release();
+  chain_wait();
   // a failed binning (instance capacity exceeded) leaves no valid lists
   if (A.hdr->status != 0) return;
   for (;;) {
@@ -622,6 +624,7 @@ __global__ void __launch_bounds__(TW* TH, 3) k_render_fwd(const RenderArgs A) {
       A.dfinal[vw.poff + pix] = D;
     }
   }
+  leave_queue(&A.hdr->queue_fwd, &A.hdr->done_fwd);
   if (P.stats) {
     unsigned long long a = n_eval, bb = n_blend;
     for (int o = 16; o > 0; o >>= 1) {
@@ -803,6 +806,8 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
   const int lane = threadIdx.x & 31;
   const RastParams& P = A.P;
   uint32_t n_eval = 0, n_blend = 0;
+  chain_release();
+  chain_wait();
   // a failed binning (instance capacity exceeded) leaves no valid lists
   if (A.hdr->status != 0) return;
   for (;;) {
@@ -1006,6 +1011,7 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
       A.dfinal[vw.poff + pix] = s.D;
     }
   }
+  leave_queue(&A.hdr->queue_fwd, &A.hdr->done_fwd);
   if (P.stats) {
     unsigned long long a = n_eval, b = n_blend;
     for (int o = 16; o > 0; o >>= 1) {
@@ -1153,6 +1159,8 @@ __global__ void __launch_bounds__(TW* TH, (TW * TH == 64) ? (CHUNK <= 64 ? 16 : 
   const RastParams& P = A.P;
   uint32_t n_eval = 0, n_blend = 0, n_outside = 0;
   uint8_t* own = S.own[wid];
+  chain_release();
+  chain_wait();
   // a failed binning (instance capacity exceeded) leaves no valid lists
   if (A.hdr->status != 0) return;
   const bool want_n = A.d_normal != nullptr;  // normal terms only when their gradient is asked for
@@ -1493,6 +1501,7 @@ __global__ void __launch_bounds__(TW* TH, (TW * TH == 64) ? (CHUNK <= 64 ? 16 : 
       restat = !restat;
     }
   }
+  leave_queue(&A.hdr->queue_bwd, &A.hdr->done_bwd);
   if (P.stats) {
     unsigned long long a = n_eval, bb = n_blend;
     for (int o = 16; o > 0; o >>= 1) {
@@ -1580,6 +1589,7 @@ __global__ void __launch_bounds__(TW* TH) k_max_error(const RenderArgs A, const 
       __syncthreads();
     }
   }
+  leave_queue(&A.hdr->queue_aux, &A.hdr->done_aux);
 }
 
 // ---------------------------------------------------------------------------
@@ -1629,9 +1639,7 @@ static cudaError_t run_fwd_k(const RenderArgs& A, cudaStream_t st) {
     grid = persistent_grid(k, TW * TH, smem, A.T);
     grid_T = A.T;
   }
-  k<<<grid, TW * TH, smem, st>>>(A);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_chained(k, grid, TW * TH, smem, st, A);
 }
 // One warp-per-tile launch: NP = 2 pixels per lane, or 1 (two items per tile).
 template <int NP, typename K>
@@ -1642,9 +1650,7 @@ static cudaError_t run_warp_kernel(K k, size_t smem, const RenderArgs& A, int64_
     grid = persistent_grid(k, WARPS * 32, smem, (items + WARPS - 1) / WARPS);
     grid_T = A.T;
   }
-  k<<<grid, WARPS * 32, smem, st>>>(A);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_chained(k, grid, WARPS * 32, smem, st, A);
 }
 template <int NP, bool RAY, bool DIST>
 static cudaError_t run_fwd_warp(const RenderArgs& A, cudaStream_t st) {
@@ -1673,9 +1679,7 @@ static cudaError_t run_bwd_k(const RenderArgs& A, cudaStream_t st) {
     grid = persistent_grid(k, TW * TH, smem, A.T);
     grid_T = A.T;
   }
-  k<<<grid, TW * TH, smem, st>>>(A);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_chained(k, grid, TW * TH, smem, st, A);
 }
 template <int TW, int TH, int CHUNK>
 static cudaError_t run_bwd(const RenderArgs& A, cudaStream_t st) {
@@ -1722,9 +1726,6 @@ cudaError_t launch_render_fwd(const Layout& L, const RastParams& P, int chunk, c
   A.normal = normal;
   A.alpha = alpha;
   A.dist = dist;
-  Header* hdr = reinterpret_cast<Header*>(ws + L.header);
-  cudaError_t e = cudaMemsetAsync(&hdr->queue_fwd, 0, sizeof(uint32_t), st);
-  if (e != cudaSuccess) return e;
   if (P.tile_w == 8 && P.tile_h == 8)
     return A.T > (int64_t)FW_WHOLE_TILES_PER_SM * sm_count() ? run_fwd_tiles8<2>(A, st) : run_fwd_tiles8<1>(A, st);
   S2D_DISPATCH(run_fwd, P.tile_w, P.tile_h, chunk, A, st);
@@ -1740,9 +1741,6 @@ cudaError_t launch_render_bwd(const Layout& L, const RastParams& P, int chunk, c
   A.d_normal = d_normal;
   A.d_alpha = d_alpha;
   A.d_dist = d_dist;
-  Header* hdr = reinterpret_cast<Header*>(ws + L.header);
-  cudaError_t e = cudaMemsetAsync(&hdr->queue_bwd, 0, sizeof(uint32_t), st);
-  if (e != cudaSuccess) return e;
   if (P.tile_w == 8 && P.tile_h == 8) {
     if (chunk == 64) return run_bwd<8, 8, 64>(A, st);
     if (chunk == 128) return run_bwd<8, 8, 128>(A, st);
@@ -1756,9 +1754,6 @@ cudaError_t launch_max_error(const Layout& L, const RastParams& P, int chunk, ch
                              const float* err, float* max_err, cudaStream_t st) {
   if (L.T <= 0) return cudaSuccess;
   RenderArgs A = make_args(L, P, ws, vals);
-  Header* hdr = reinterpret_cast<Header*>(ws + L.header);
-  cudaError_t e = cudaMemsetAsync(&hdr->queue_aux, 0, sizeof(uint32_t), st);
-  if (e != cudaSuccess) return e;
   uint32_t* m = reinterpret_cast<uint32_t*>(max_err);
   if (P.tile_w == 8 && P.tile_h == 8) return run_max_error<8, 8>(A, err, m, st);
   if (P.tile_w == 16 && P.tile_h == 16) return run_max_error<16, 16>(A, err, m, st);

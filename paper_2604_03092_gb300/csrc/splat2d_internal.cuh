@@ -53,7 +53,8 @@ struct Header {
   uint32_t queue_fwd, queue_bwd; // persistent work queues
   unsigned long long stat[8];    // pair counters, see STAT_*
   uint32_t queue_aux;            // work queue of the error-attribution pass
-  uint32_t pad[31];
+  uint32_t done_fwd, done_bwd, done_aux;  // CTAs that have left each queue's kernel
+  uint32_t pad[28];
 };
 static_assert(sizeof(Header) <= 256, "Header layout");
 enum { STAT_FWD_EVAL = 0, STAT_FWD_BLEND = 1, STAT_BWD_EVAL = 2, STAT_BWD_BLEND = 3, STAT_BWD_OUTSIDE = 4 };
@@ -93,6 +94,7 @@ struct Layout {
   int64_t bmask_words;  // 32-entry words of blended-pair masks (each holds one word per tile pixel)
   int64_t R, T, P, cap;
   int64_t n_work;     // sum over view groups of the surfel range sizes
+  int64_t max_range;  // the longest view's surfel range
   int32_t V, G;
   bool groups_overlap;  // some surfel belongs to two groups
   int32_t sort_blocks;
@@ -103,7 +105,8 @@ constexpr int SORT_THREADS = 256;
 constexpr int SORT_IPT = 8;
 constexpr int SORT_TILE = SORT_THREADS * SORT_IPT;  // 2048 keys per tile
 constexpr int SORT_MAX_BLOCKS = 1024;
-constexpr int ORDER_BINS = 64;   // cost buckets of the work queue order
+constexpr int ORDER_BINS = 33;   // cost buckets of the work queue order: bit lengths 32..0
+constexpr int TILE_HIST_WORDS = 80;  // small counters of the binning (see launch_bin_tiles)
 
 __host__ __device__ __forceinline__ int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
 __host__ __device__ __forceinline__ int64_t max64(int64_t a, int64_t b) { return a > b ? a : b; }
@@ -127,11 +130,10 @@ struct RastParams {
 // ---------------------------------------------------------------------------
 // Launch wrappers (defined in the .cu files)
 // ---------------------------------------------------------------------------
-cudaError_t launch_upload(const void* host_src, size_t bytes, void* dst, cudaStream_t st);
+cudaError_t launch_setup(const void* tables, size_t table_bytes, const Layout& L, char* ws, cudaStream_t st);
 cudaError_t launch_preprocess(const splat2d_surfels* S, const Layout& L, const RastParams& P, char* ws,
                               cudaStream_t st);
 cudaError_t launch_bin_tiles(const Layout& L, const RastParams& P, char* ws, cudaStream_t st);
-cudaError_t launch_order(const Layout& L, char* ws, cudaStream_t st);
 cudaError_t launch_sort(uint64_t* keys0, uint32_t* vals0, uint64_t* keys1, uint32_t* vals1,
                         const unsigned long long* n_dev, int64_t n_max, int key_bits, uint32_t* hist,
                         int sort_blocks, int* final_buffer, cudaStream_t st);
@@ -160,6 +162,32 @@ void count_launches(int n);  // host-side tally of kernels enqueued
 // Device helpers
 // ---------------------------------------------------------------------------
 #ifdef __CUDACC__
+
+// Kernels of one step are launched so that a kernel's blocks may be scheduled
+// while the kernel before it still runs (programmatic dependent launch): each
+// lets the next one start, then waits until the one before has completed and
+// its writes are visible.  As every kernel waits, completion is transitive,
+// and a launch that is not chained waits for all of them as usual.  It takes
+// the launch latency out of the gaps: see launch_bin_tiles for what it gave.
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... K, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(K...), int grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, K(args)...);
+  count_launches(1);
+  return e;
+}
 
 // Error-free transformations (Knuth's TwoSum; the FMA-based exact product).
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -218,6 +246,17 @@ __device__ __forceinline__ float2 unpack_half2_scaled(uint32_t u) {
   __half2 h = *reinterpret_cast<__half2*>(&u);
   float2 f = __half22float2(h);
   return make_float2(f.x * (1.0f / 65536.0f), f.y * (1.0f / 65536.0f));
+}
+
+// Leaves a persistent kernel's work queue: the last CTA to leave sets it (and
+// the count of those that left) back to zero for the kernel's next launch.
+// Every thread calls it, once, after the CTA's last item.
+__device__ __forceinline__ void leave_queue(uint32_t* queue, uint32_t* done) {
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(done, 1u) == gridDim.x - 1) {
+    *queue = 0u;
+    *done = 0u;
+  }
 }
 
 // Index of the view owning global tile `t` (views sorted by tile_base).
