@@ -305,6 +305,15 @@ int splat2d_render_bwd_tiles_dist(const splat2d_config* cfg, const splat2d_probl
                                   const float* d_alpha, const float* d_dist, splat2d_stream stream);
 
 /*
+ * splat2d_preprocess, splat2d_bin_sort and splat2d_render_fwd_dist on one
+ * workspace, in this order, in one call (the arguments are checked and the
+ * tables built once).  Errors as for the three.
+ */
+int splat2d_forward(const splat2d_config* cfg, const splat2d_problem* prob, const splat2d_surfels* surfels, void* ws,
+                    size_t ws_bytes, float* rgb, float* depth, float* normal, float* alpha, float* dist,
+                    splat2d_stream stream);
+
+/*
  * Map fusion, pruning input (Sec. 4.3, "Map Fusion": the global map is
  * rendered at the new keyframe's pose and primitives that contribute to
  * pixels with high RGB or depth error are removed).  For every (pixel,

@@ -94,6 +94,9 @@ SIGNATURES = {
     "splat2d_preprocess_bwd": (ctypes.c_int, [ctypes.POINTER(Config), ctypes.POINTER(Problem),
                                               ctypes.POINTER(Surfels), c_void_p, c_size_t, ctypes.POINTER(Grads),
                                               c_void_p]),
+    "splat2d_forward": (ctypes.c_int, [ctypes.POINTER(Config), ctypes.POINTER(Problem), ctypes.POINTER(Surfels),
+                                       c_void_p, c_size_t, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p,
+                                       c_void_p]),
     "splat2d_max_error": (ctypes.c_int, [ctypes.POINTER(Config), ctypes.POINTER(Problem), c_void_p, c_size_t,
                                          c_void_p, c_void_p, c_void_p]),
     "splat2d_accum_gate_tmp_size": (c_size_t, [c_int64]),

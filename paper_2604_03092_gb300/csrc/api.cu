@@ -1,6 +1,7 @@
 // C ABI of libsplat2d: argument checks, workspace layout and the launch
 // sequence of each call.  See include/splat2d.h for the contract.
 #include <cuda_runtime.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <atomic>
@@ -209,13 +210,35 @@ static RastParams make_params(const splat2d_config* c) {
 }
 
 static int check_common(const splat2d_config* cfg, const splat2d_problem* prob, void* ws, size_t ws_bytes,
-                        Layout* L) {
+                        Layout* L, HostTables* H = nullptr) {
   if (!valid_config(cfg)) return SPLAT2D_ERR_INVALID_ARG;
-  if (!build_tables(cfg, prob, L, nullptr)) return SPLAT2D_ERR_INVALID_ARG;
+  if (!build_tables(cfg, prob, L, H)) return SPLAT2D_ERR_INVALID_ARG;
   if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255)) return SPLAT2D_ERR_INVALID_ARG;
   if (ws_bytes < L->total) return SPLAT2D_ERR_WORKSPACE_TOO_SMALL;
   return SPLAT2D_OK;
 }
+
+// A thread's page-locked block for the status header (256 bytes, given back
+// when the thread ends, in the process that took it; usable from every device).
+struct PinnedHeader {
+  Header* p = nullptr;
+  bool tried = false;
+  pid_t owner = 0;
+  Header* get() {
+    if (!tried) {
+      tried = true;
+      owner = getpid();
+      if (cudaHostAlloc(reinterpret_cast<void**>(&p), sizeof(Header), cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        p = nullptr;
+      }
+    }
+    return p;
+  }
+  ~PinnedHeader() {
+    if (p && owner == getpid()) cudaFreeHost(p);
+  }
+};
 
 // The binning leaves the sorted instances in buffer 0.
 static int final_sorted_buffer(const Layout&) { return 0; }
@@ -264,20 +287,8 @@ int splat2d_workspace_layout(const splat2d_config* cfg, const splat2d_problem* p
   return SPLAT2D_OK;
 }
 
-int splat2d_preprocess(const splat2d_config* cfg, const splat2d_problem* prob, const splat2d_surfels* surfels,
-                       void* ws, size_t ws_bytes, splat2d_stream stream) {
-  Layout L;
-  int rc = check_common(cfg, prob, ws, ws_bytes, &L);
-  if (rc) return rc;
-  if (!surfels || surfels->n != prob->n_surfels) return SPLAT2D_ERR_INVALID_ARG;
-  if (prob->n_surfels > 0 && (!surfels->means || !surfels->scales || !surfels->quats || !surfels->opacity ||
-                              !surfels->rgb))
-    return SPLAT2D_ERR_INVALID_ARG;
-  if (reinterpret_cast<uintptr_t>(surfels->quats) & 15) return SPLAT2D_ERR_INVALID_ARG;
-  HostTables H;
-  build_tables(cfg, prob, &L, &H);
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  char* w = static_cast<char*>(ws);
+static int preprocess_checked(const splat2d_config* cfg, const splat2d_surfels* surfels, const Layout& L,
+                              const HostTables& H, char* w, cudaStream_t st) {
   // the header (zero), the views and the groups as they lie in the workspace
   const size_t table_bytes = L.groups + sizeof(DGroup) * H.groups.size() - L.header;
   std::vector<char> tables(table_bytes, 0);
@@ -285,9 +296,28 @@ int splat2d_preprocess(const splat2d_config* cfg, const splat2d_problem* prob, c
   if (!H.groups.empty())
     std::memcpy(tables.data() + (L.groups - L.header), H.groups.data(), sizeof(DGroup) * H.groups.size());
   if (launch_setup(tables.data(), table_bytes, L, w, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
-  RastParams P = make_params(cfg);
-  if (launch_preprocess(surfels, L, P, w, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+  if (launch_preprocess(surfels, L, make_params(cfg), w, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
   return SPLAT2D_OK;
+}
+
+static int check_surfels(const splat2d_problem* prob, const splat2d_surfels* surfels) {
+  if (!surfels || surfels->n != prob->n_surfels) return SPLAT2D_ERR_INVALID_ARG;
+  if (prob->n_surfels > 0 && (!surfels->means || !surfels->scales || !surfels->quats || !surfels->opacity ||
+                              !surfels->rgb))
+    return SPLAT2D_ERR_INVALID_ARG;
+  if (reinterpret_cast<uintptr_t>(surfels->quats) & 15) return SPLAT2D_ERR_INVALID_ARG;
+  return SPLAT2D_OK;
+}
+
+int splat2d_preprocess(const splat2d_config* cfg, const splat2d_problem* prob, const splat2d_surfels* surfels,
+                       void* ws, size_t ws_bytes, splat2d_stream stream) {
+  Layout L;
+  HostTables H;
+  int rc = check_common(cfg, prob, ws, ws_bytes, &L, &H);
+  if (rc) return rc;
+  rc = check_surfels(prob, surfels);
+  if (rc) return rc;
+  return preprocess_checked(cfg, surfels, L, H, static_cast<char*>(ws), reinterpret_cast<cudaStream_t>(stream));
 }
 
 int splat2d_bin_sort(const splat2d_config* cfg, const splat2d_problem* prob, void* ws, size_t ws_bytes,
@@ -295,10 +325,18 @@ int splat2d_bin_sort(const splat2d_config* cfg, const splat2d_problem* prob, voi
   Layout L;
   int rc = check_common(cfg, prob, ws, ws_bytes, &L);
   if (rc) return rc;
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  char* w = static_cast<char*>(ws);
-  RastParams P = make_params(cfg);
-  if (launch_bin_tiles(L, P, w, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+  if (launch_bin_tiles(L, make_params(cfg), static_cast<char*>(ws), reinterpret_cast<cudaStream_t>(stream)) !=
+      cudaSuccess)
+    return SPLAT2D_ERR_CUDA;
+  return SPLAT2D_OK;
+}
+
+static int render_fwd_checked(const splat2d_config* cfg, const Layout& L, char* w, float* rgb, float* depth,
+                              float* normal, float* alpha, float* dist, cudaStream_t st) {
+  const uint32_t* vals = reinterpret_cast<const uint32_t*>(w + (final_sorted_buffer(L) ? L.vals1 : L.vals0));
+  if (launch_render_fwd(L, make_params(cfg), cfg->chunk, w, vals, rgb, depth, normal, alpha, dist, st) !=
+      cudaSuccess)
+    return SPLAT2D_ERR_CUDA;
   return SPLAT2D_OK;
 }
 
@@ -308,13 +346,25 @@ int splat2d_render_fwd_dist(const splat2d_config* cfg, const splat2d_problem* pr
   Layout L;
   int rc = check_common(cfg, prob, ws, ws_bytes, &L);
   if (rc) return rc;
+  return render_fwd_checked(cfg, L, static_cast<char*>(ws), rgb, depth, normal, alpha, dist,
+                            reinterpret_cast<cudaStream_t>(stream));
+}
+
+int splat2d_forward(const splat2d_config* cfg, const splat2d_problem* prob, const splat2d_surfels* surfels, void* ws,
+                    size_t ws_bytes, float* rgb, float* depth, float* normal, float* alpha, float* dist,
+                    splat2d_stream stream) {
+  Layout L;
+  HostTables H;
+  int rc = check_common(cfg, prob, ws, ws_bytes, &L, &H);
+  if (rc) return rc;
+  rc = check_surfels(prob, surfels);
+  if (rc) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
-  const uint32_t* vals = reinterpret_cast<const uint32_t*>(w + (final_sorted_buffer(L) ? L.vals1 : L.vals0));
-  if (launch_render_fwd(L, make_params(cfg), cfg->chunk, w, vals, rgb, depth, normal, alpha, dist, st) !=
-      cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
-  return SPLAT2D_OK;
+  rc = preprocess_checked(cfg, surfels, L, H, w, st);
+  if (rc) return rc;
+  if (launch_bin_tiles(L, make_params(cfg), w, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+  return render_fwd_checked(cfg, L, w, rgb, depth, normal, alpha, dist, st);
 }
 
 int splat2d_render_fwd(const splat2d_config* cfg, const splat2d_problem* prob, void* ws, size_t ws_bytes,
@@ -349,11 +399,9 @@ int splat2d_preprocess_bwd(const splat2d_config* cfg, const splat2d_problem* pro
   Layout L;
   int rc = check_common(cfg, prob, ws, ws_bytes, &L);
   if (rc) return rc;
-  if (!surfels || surfels->n != prob->n_surfels || !grads) return SPLAT2D_ERR_INVALID_ARG;
-  if (prob->n_surfels > 0 && (!surfels->means || !surfels->scales || !surfels->quats || !surfels->opacity ||
-                              !surfels->rgb))
-    return SPLAT2D_ERR_INVALID_ARG;
-  if (reinterpret_cast<uintptr_t>(surfels->quats) & 15) return SPLAT2D_ERR_INVALID_ARG;
+  if (!grads) return SPLAT2D_ERR_INVALID_ARG;
+  rc = check_surfels(prob, surfels);
+  if (rc) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (launch_preprocess_bwd(surfels, L, make_params(cfg), static_cast<char*>(ws), grads, L.groups_overlap, st) !=
       cudaSuccess)
@@ -438,9 +486,19 @@ uint64_t splat2d_launch_count(void) { return s2d::launch_counter().load(); }
 int splat2d_stats(const void* ws, splat2d_stats_t* out, splat2d_stream stream) {
   if (!ws || !out) return SPLAT2D_ERR_INVALID_ARG;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (cudaStreamSynchronize(st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+  // the copy runs on the stream, into this thread's page-locked block: one
+  // wait instead of a wait and a blocking copy
+  static thread_local PinnedHeader pinned;
+  Header* dst = pinned.get();
   Header h;
-  if (cudaMemcpy(&h, ws, sizeof(Header), cudaMemcpyDeviceToHost) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+  if (dst) {
+    if (cudaMemcpyAsync(dst, ws, sizeof(Header), cudaMemcpyDeviceToHost, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+    if (cudaStreamSynchronize(st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+    h = *dst;
+  } else {
+    if (cudaStreamSynchronize(st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+    if (cudaMemcpy(&h, ws, sizeof(Header), cudaMemcpyDeviceToHost) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+  }
   std::memset(out, 0, sizeof(*out));
   out->status = h.status;
   out->needed_capacity = (int64_t)h.needed;

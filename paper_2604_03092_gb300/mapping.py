@@ -35,7 +35,7 @@ def voxelize(means, quats, scales, opacity, rgb, width: int, height: int, tau_d:
     dev = means.device
     out = [torch.empty_like(t) for t in ins]
     block = torch.empty(max(n, 1), dtype=torch.int32, device=dev)
-    n_out = torch.zeros(1, dtype=torch.int64, device=dev)
+    n_out = torch.empty(1, dtype=torch.int64, device=dev)  # written whatever the size is
     tmp = torch.empty(max(int(lib.splat2d_voxelize_tmp_size(width, height)), 4), dtype=torch.uint8, device=dev)
     sf = _abi.Surfels(*[t.data_ptr() for t in ins], n)
     ob = _abi.SurfelBuffers(*[t.data_ptr() for t in out])

@@ -93,7 +93,9 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    """The current device's current stream (the raw handle: building a
+    torch.cuda.Stream around it costs more than a launch)."""
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 class Rasterizer:
@@ -309,14 +311,19 @@ class Rasterizer:
 
     def forward(self, means, scales, quats, opacity, rgb, out: Optional[Images] = None, check: bool = True,
                 max_retries: int = 3, dist: Optional[torch.Tensor] = None) -> Images:
-        """preprocess -> bin_sort -> render_fwd.  With check=True the device
+        """preprocess -> bin_sort -> render_fwd, in one call of the library.  With check=True the device
         status is read (a synchronisation) and an instance-capacity overflow
         is repaired by growing the workspace and running again."""
         out = out or self.new_images()
+        if means.shape[0] != self.n_surfels:
+            raise ValueError(f"expected {self.n_surfels} surfels, got {means.shape[0]}")
         for _ in range(max_retries + 1):
-            self.preprocess(means, scales, quats, opacity, rgb)
-            self.bin_sort()
-            self.render_fwd(out, dist)
+            self.generation += 1
+            self._sf = self._surfels(means, scales, quats, opacity, rgb)
+            _abi.check(self.lib.splat2d_forward(ctypes.byref(self._cfg), ctypes.byref(self._prob),
+                                                ctypes.byref(self._sf), self._ws_ptr, self.ws_bytes, _ptr(out.rgb),
+                                                _ptr(out.depth), _ptr(out.normal), _ptr(out.alpha), _ptr(dist),
+                                                _stream()), "splat2d_forward")
             if not check:
                 return out
             rc = self.status()
@@ -329,8 +336,10 @@ class Rasterizer:
 
     def new_grads(self) -> SurfelGrads:
         n, dev = self.n_surfels, self.device
-        z = lambda *s: torch.zeros(*s, device=dev)
-        return SurfelGrads(z(n, 3), z(n, 2), z(n, 4), z(n), z(n, 3), z(self.n_views, 6))
+        e = lambda *s: torch.empty(*s, device=dev)
+        g = SurfelGrads(e(n, 3), e(n, 2), e(n, 4), e(n), e(n, 3), e(self.n_views, 6))
+        torch._foreach_zero_(list(g))  # one launch
+        return g
 
     def backward(self, means, scales, quats, opacity, rgb, d_out: Sequence[Optional[torch.Tensor]],
                  grads: Optional[SurfelGrads] = None, d_dist: Optional[torch.Tensor] = None) -> SurfelGrads:
@@ -355,7 +364,7 @@ def accum_gate(alpha: torch.Tensor, tau: float):
         raise ValueError("alpha: float32 CUDA tensor")
     n = alpha.numel()
     keep = torch.empty(max(n, 1), dtype=torch.int32, device=alpha.device)
-    n_keep = torch.zeros(1, dtype=torch.int64, device=alpha.device)
+    n_keep = torch.empty(1, dtype=torch.int64, device=alpha.device)  # written whatever n is
     tmp = torch.empty(max(int(lib.splat2d_accum_gate_tmp_size(n)), 4), dtype=torch.uint8, device=alpha.device)
     _abi.check(lib.splat2d_accum_gate(_ptr(alpha), n, float(tau), keep.data_ptr(), n_keep.data_ptr(),
                                       tmp.data_ptr(), tmp.numel(), _stream()), "splat2d_accum_gate")
@@ -367,8 +376,8 @@ class Splat2DRender(torch.autograd.Function):
     normal, alpha).
 
     `pose_tangent` ([V, 6]) receives dL/dxi of each view's pose under the
-    left perturbation T_cw <- Exp(xi) T_cw, evaluated at xi = 0.  Its value
-    does not enter the render: the poses are the rasterizer's views, so a
+    left perturbation T_cw <- Exp(xi) T_cw, evaluated at xi = 0 (None: not
+    asked for).  Its value does not enter the render: the poses are the rasterizer's views, so a
     caller that refines poses folds each step into them
     (`Rasterizer.set_view_pose`) and keeps xi at zero.
 
@@ -380,6 +389,7 @@ class Splat2DRender(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, rast: Rasterizer, means, scales, quats, opacity, rgb, pose_tangent, check: bool = True):
+        ctx.set_materialize_grads(False)  # an output without a gradient costs the backward nothing
         params = [t.contiguous() for t in (means, scales, quats, opacity, rgb)]
         out = rast.forward(*params, check=check)
         ctx.rast = rast
@@ -397,7 +407,8 @@ class Splat2DRender(torch.autograd.Function):
                                "render that is differentiated")
         params = ctx.saved_tensors
         grads = rast.backward(*params, (g_rgb, g_depth, g_normal, g_alpha))
-        return (None, grads.means, grads.scales, grads.quats, grads.opacity, grads.rgb, grads.pose, None)
+        return (None, grads.means, grads.scales, grads.quats, grads.opacity, grads.rgb,
+                grads.pose if ctx.needs_input_grad[6] else None, None)
 
 
 class Splat2DRenderDist(torch.autograd.Function):
@@ -407,6 +418,7 @@ class Splat2DRenderDist(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, rast: Rasterizer, means, scales, quats, opacity, rgb, pose_tangent, check: bool = True):
+        ctx.set_materialize_grads(False)
         params = [t.contiguous() for t in (means, scales, quats, opacity, rgb)]
         dist = torch.empty(rast.n_pixels, device=rast.device)
         out = rast.forward(*params, check=check, dist=dist)
@@ -428,14 +440,13 @@ class Splat2DRenderDist(torch.autograd.Function):
                                "render that is differentiated")
         params = ctx.saved_tensors
         grads = rast.backward(*params, (g_rgb, g_depth, g_normal, g_alpha), d_dist=g_dist)
-        return (None, grads.means, grads.scales, grads.quats, grads.opacity, grads.rgb, grads.pose, None)
+        return (None, grads.means, grads.scales, grads.quats, grads.opacity, grads.rgb,
+                grads.pose if ctx.needs_input_grad[6] else None, None)
 
 
 def render(rast: Rasterizer, means, scales, quats, opacity, rgb, pose_tangent=None, check: bool = True,
            distortion: bool = False):
     """Functional form of Splat2DRender (with distortion=True, of
     Splat2DRenderDist: the depth distortion map is a fifth output)."""
-    if pose_tangent is None:
-        pose_tangent = torch.zeros(rast.n_views, 6, device=means.device, requires_grad=False)
     fn = Splat2DRenderDist if distortion else Splat2DRender
     return fn.apply(rast, means, scales, quats, opacity, rgb, pose_tangent, check)
