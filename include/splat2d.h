@@ -119,7 +119,7 @@ typedef struct {
 typedef struct {
   int32_t tile_w, tile_h;   /* one of 8x8, 16x16, 32x8 */
   int32_t chunk;            /* surfels staged per shared-memory batch: 64, 128, 256 (or 512 with 256-pixel tiles); the
-                               forward of 8x8 tiles stages 32 whatever it says */
+                               forward of 8x8 tiles stages 32, and this many in a tile's tail (see below) */
   float alpha_min;          /* skip pairs with alpha below this */
   float alpha_max;          /* clamp of alpha (keeps the reverse pass finite) */
   float t_min;              /* stop a pixel before T would drop below this */
@@ -143,7 +143,7 @@ typedef struct {
  * which the forward shares the tile's remaining pixels across all warps
  * (0 = the default of 6; 255 = always).  A launch-shape knob for the
  * autotuner: it changes the schedule, not the result beyond rounding.  8x8
- * tiles are composited by one warp each and ignore it. */
+ * tiles are handed to a second kernel from that chunk on. */
 #define SPLAT2D_FLAG_TAIL_SHIFT 8
 
 /* The shape of one problem: the views (host array) and sizes.  Pass the same

@@ -213,6 +213,8 @@ struct RenderArgs {
   const float* d_depth;
   const float* d_normal;
   const float* d_alpha;
+  int32_t chunk;        // forward: list entries per chunk
+  uint2* tails;         // forward, 8x8 tiles: tile and list index from which k_render_tail goes on
 };
 
 // Copies entries [base, base + count) of the sorted list's records to shared
@@ -642,8 +644,8 @@ __global__ void __launch_bounds__(TW* TH, 3) k_render_fwd(const RenderArgs A) {
 // Forward for 8x8 tiles
 // ---------------------------------------------------------------------------
 // One warp per tile (NP = 2), or per half of a tile (NP = 1: four rows; where
-// there are too few tiles to fill the GPU), no block barriers.  The tile's
-// list is taken 32 entries at a time, in two passes:
+// there are too few tiles to fill the GPU), no block barriers, until few of
+// its pixels are left (k_render_tail).  The tile's list is taken 32 entries at a time, in two passes:
 //   1. entry-major: each lane owns an entry, its record in registers, and
 //      evaluates alpha at the active pixels of its rect (a bit mask), two per
 //      step in packed FP32; alphas of at least alpha_min go to a pixel x entry
@@ -660,9 +662,9 @@ __global__ void __launch_bounds__(TW* TH, 3) k_render_fwd(const RenderArgs A) {
 // all lanes together instead.
 // Issue-bound (71% of the issue slots on 4 keyframes x 4 views); the blending
 // pass keeps 17% of its lanes busy where many keyframes overlap, 41% on one.
-// 24 keyframes x 24 views at 512x384: 16.3 -> 11.0 ms; one keyframe x 8 views
-// 557 -> 440 us.
-constexpr int WARPS = 4;       // warps per CTA of the warp-per-tile kernels; they share nothing
+// With k_render_tail, against k_render_fwd for all of it: 24 keyframes x 24
+// views at 512x384 16.3 -> 12.2 ms; one keyframe x 8 views 557 -> 465 us.
+constexpr int WARPS = 4;       // warps per CTA of the warp-per-tile forward
 constexpr int FW_STRIDE = 33;  // floats per pixel row of the alpha table
 // (pixel, entry) pairs per 32 pixels (of 1024) that make a chunk dense: two
 // 333x251 views of 20 K large surfels 157 us without the dense walk, 129 with
@@ -670,10 +672,12 @@ constexpr int FW_STRIDE = 33;  // floats per pixel row of the alpha table
 constexpr uint32_t FW_DENSE = 350;
 // Up to this many tiles per SM a warp takes half a tile: twice the warps, and
 // a shorter chain per chunk, where the tiles are too few for whole ones to
-// keep the SM's 24 warps busy.  Whole against half, 8 keyframes in one view:
-// 300 tiles 1319 / 921 us, 1900 tiles 365 / 290, 3072 tiles 344 / 293; one
-// keyframe, 3072 tiles 83 / 88; 7260 tiles 317 / 308; 24576 tiles 440 / 499.
-constexpr int FW_WHOLE_TILES_PER_SM = 32;
+// keep the SM's 24 warps busy.  Whole against half, one keyframe in one view:
+// 300 tiles 186 / 144 us, 1200 88 / 80, 1938 88 / 98, 3072 97 / 117, 4800
+// 117 / 133; 8 keyframes: 300 tiles 1349 / 1052, 1200 511 / 401, 1938 429 /
+// 423, 3072 434 / 440, 4800 409 / 497; 2688 tiles of large surfels (dense
+// chunks) 148 / 106.
+constexpr int FW_WHOLE_TILES_PER_SM = 18;
 
 template <int NP>
 struct FwdWarpBase {
@@ -747,6 +751,32 @@ __device__ __forceinline__ bool any_bits(const uint32_t (&m)[NP]) {
   return (m[0] | m[NP - 1]) != 0u;
 }
 
+// Records of 32 list entries (lane e gives the e-th one's record number, or
+// ~0: none), as float4 number lane + 32 k of theirs: five neighbouring lanes
+// take one record's five float4, so a load instruction touches the lines of
+// seven records (a lane per record touches 32, five times over: that bound the
+// gather on L1 tag lookups) and a store to the sorted-order copy is contiguous.
+__device__ __forceinline__ void load_records(const RenderArgs& A, uint32_t ri, int lane, float4 (&f)[REC_F4]) {
+#pragma unroll
+  for (int k = 0; k < REC_F4; k++) {
+    const int i = lane + 32 * k, e = (i * 205) >> 10;  // i / 5 for i < 160
+    const uint32_t r = __shfl_sync(0xffffffffu, ri, e);
+    f[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r != 0xffffffffu) f[k] = __ldg(A.records + (size_t)r * REC_F4 + (i - 5 * e));
+  }
+}
+// ... to shared memory and, the first `count`, to the copy the backward reads
+// (streaming stores, read long after); `base`: the first one's list index.
+__device__ __forceinline__ void store_records(const RenderArgs& A, int64_t base, int count, int lane,
+                                              const float4 (&f)[REC_F4], float4* raw) {
+#pragma unroll
+  for (int k = 0; k < REC_F4; k++) {
+    const int i = lane + 32 * k;
+    raw[i] = f[k];
+    if (i < count * REC_F4) __stcs(A.rcopy + base * REC_F4 + i, f[k]);
+  }
+}
+
 // One pixel's compositing state.
 template <bool DIST>
 struct PixelSums {
@@ -797,12 +827,34 @@ __device__ __forceinline__ uint32_t blend_pixel(const FwdWarpSmem<NP, RAY>& S, i
   return todo;
 }
 
+// Where a warp takes half a tile, its neighbour takes the other: both get the
+// sum of the numbers that their lanes 0 give.  Two slots by turns: a warp
+// writes a slot again only after the barrier of the turn in between, which the
+// other one reaches after having read it.
+template <bool USED>
+struct HalfPairs {
+  uint32_t slot[USED ? WARPS / 2 : 1][2][2];
+  __device__ __forceinline__ uint32_t sum(uint32_t x, uint32_t& turn) {
+    const int pair = threadIdx.x >> 6, half = (threadIdx.x >> 5) & 1;
+    volatile uint32_t* s = slot[pair][turn];
+    turn ^= 1u;
+    if ((threadIdx.x & 31) == 0) s[half] = x;
+    asm volatile("bar.sync %0, 64;" ::"r"(pair + 1) : "memory");
+    return s[0] + s[1];
+  }
+};
+
+// A tile of which at most fwd_tail pixels per 32 are still compositing at the
+// start of a chunk (of A.chunk entries, counted from the tile's first) is
+// handed over to k_render_tail, its pixels' state in the images.
 // 80 registers: 6 CTAs (24 warps) per SM, as many as the alpha tables leave
 // room for (NP = 2).
 template <int NP, bool RAY, bool DIST>
 __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(const RenderArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   FwdWarpSmem<NP, RAY>& S = reinterpret_cast<FwdWarpSmem<NP, RAY>*>(smem_raw)[threadIdx.x >> 5];
+  __shared__ HalfPairs<NP == 1> pairs_of_halves;
+  uint32_t turn = 0;
   const int lane = threadIdx.x & 31;
   const RastParams& P = A.P;
   uint32_t n_eval = 0, n_blend = 0;
@@ -812,10 +864,10 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
   if (A.hdr->status != 0) return;
   for (;;) {
     uint32_t item = 0;
-    if (lane == 0) item = atomicAdd(&A.hdr->queue_fwd, 1u);
-    item = __shfl_sync(0xffffffffu, item, 0);
-    const int half = NP == 1 ? (int)(item & 1u) : 0;
-    if (NP == 1) item >>= 1;
+    const int half = NP == 1 ? (threadIdx.x >> 5) & 1 : 0;
+    if (lane == 0 && half == 0) item = atomicAdd(&A.hdr->queue_fwd, 1u);
+    if constexpr (NP == 1) item = pairs_of_halves.sum(item, turn);
+    else item = __shfl_sync(0xffffffffu, item, 0);
     if ((int64_t)item >= A.T) break;
     const int t = (int)__ldg(A.order + item);
     const int v = find_view_by_tile(A.views, A.V, t);
@@ -838,38 +890,36 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
     // this lane's list entry of the chunk staged next, read one chunk ahead
     uint32_t ent = range.x + lane < range.y ? __ldg(A.vals + range.x + lane) : 0u;
     uint32_t word = (range.x >> 5) + (uint32_t)t;  // the chunk's blended-mask word
+    bool tail = false;
     for (int64_t base = range.x; base < range.y; base += 32, word++) {
       uint32_t live_px[NP];
 #pragma unroll
       for (int h = 0; h < NP; h++) live_px[h] = __ballot_sync(0xffffffffu, !done[h]);
-      if (!any_bits<NP>(live_px)) break;
+      if ((((uint32_t)base - range.x) & (uint32_t)(A.chunk - 1)) == 0u) {
+        uint32_t n_act = count_bits<NP>(live_px);
+        if constexpr (NP == 1) n_act = pairs_of_halves.sum(n_act, turn);
+        if (n_act == 0) break;
+        if ((int)n_act <= P.fwd_tail * 2) {
+          if (lane == 0 && half == 0) __stcg(A.tails + atomicAdd(&A.hdr->n_tails, 1u), make_uint2((uint32_t)t, (uint32_t)base));
+          tail = true;
+          break;
+        }
+      }
+      if (!any_bits<NP>(live_px)) {
+        if (NP == 1) continue;  // up to the next chunk, for the other half
+        break;
+      }
       const int count = (int)min64(32, (int64_t)range.y - base);
       const uint32_t sf = ent;
       ent = base + 32 + lane < (int64_t)range.y ? __ldg(A.vals + base + 32 + lane) : 0u;
       const bool ok =
           lane < count && s2d_check((int64_t)sf >= vw.soff && (int64_t)sf < vw.soff + vw.scnt, A.hdr);
       const uint32_t ri = ok ? (uint32_t)(vw.rbase + ((int64_t)sf - vw.soff)) : 0xffffffffu;
-      // gather the chunk's records: five neighbouring lanes take one record's
-      // five float4, so a load instruction touches the lines of seven records
-      // (a lane per record touches 32, five times over: that bound the gather
-      // on L1 tag lookups) and a store to the sorted-order copy is contiguous
       float4* raw = reinterpret_cast<float4*>(S.alpha);  // until pass 1 writes alphas there
       {
         float4 f[REC_F4];
-#pragma unroll
-        for (int k = 0; k < REC_F4; k++) {
-          const int i = lane + 32 * k, e = (i * 205) >> 10;  // i / 5 for i < 160
-          const uint32_t r = __shfl_sync(0xffffffffu, ri, e);
-          f[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (r != 0xffffffffu) f[k] = __ldg(A.records + (size_t)r * REC_F4 + (i - 5 * e));
-        }
-#pragma unroll
-        for (int k = 0; k < REC_F4; k++) {
-          const int i = lane + 32 * k;
-          raw[i] = f[k];
-          // the backward reads the records in list order; streaming stores, read long after
-          if (i < count * REC_F4) __stcs(A.rcopy + base * REC_F4 + i, f[k]);
-        }
+        load_records(A, ri, lane, f);
+        store_records(A, base, count, lane, f, raw);
       }
       __syncwarp();
       float4 c = make_float4(0.f, 0.f, 0.f, 0.f), p = c, q = c;
@@ -993,9 +1043,9 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
       const int64_t pix = (int64_t)(ipy + 4 * h) * vw.W + ipx;
       if (A.rgb) {
         float* o = A.rgb + 3 * vw.poff + pix;
-        o[0] = __fmaf_rn(s.T, P.bg[0], s.C0);
-        o[HW] = __fmaf_rn(s.T, P.bg[1], s.C1);
-        o[2 * HW] = __fmaf_rn(s.T, P.bg[2], s.C2);
+        o[0] = tail ? s.C0 : __fmaf_rn(s.T, P.bg[0], s.C0);
+        o[HW] = tail ? s.C1 : __fmaf_rn(s.T, P.bg[1], s.C1);
+        o[2 * HW] = tail ? s.C2 : __fmaf_rn(s.T, P.bg[2], s.C2);
       }
       if (A.depth) A.depth[vw.poff + pix] = s.D;
       if (A.normal) {
@@ -1006,12 +1056,249 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
       }
       if (A.alpha) A.alpha[vw.poff + pix] = 1.f - s.T;
       if constexpr (DIST) A.dist[vw.poff + pix] = s.Ds;
-      A.tfinal[vw.poff + pix] = s.T;
+      A.tfinal[vw.poff + pix] = tail && done[h] ? -s.T : s.T;
       A.last[vw.poff + pix] = last[h];
       A.dfinal[vw.poff + pix] = s.D;
     }
   }
   leave_queue(&A.hdr->queue_fwd, &A.hdr->done_fwd);
+  if (P.stats) {
+    unsigned long long a = n_eval, b = n_blend;
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if (lane == 0) {
+      atomicAdd(&A.hdr->stat[STAT_FWD_EVAL], a);
+      atomicAdd(&A.hdr->stat[STAT_FWD_BLEND], b);
+    }
+  }
+}
+
+// The tail of the 8x8 tiles that k_render_fwd_warp has handed over: a warp
+// composites 32 of a pixel's entries per step with a prefix product of
+// (1 - alpha), as k_render_fwd does below the same number of pixels, whose
+// rounding the stop at t_min and the backward's fixed-point terms depend on (a
+// product front to back instead moved single gradients by 2e-3).
+// Few tiles get here, with long lists, so it is bound by the chain of chunks:
+// a warp per 32 entries of the chunk, the next chunk's records read while this
+// one's are composited, and each pixel's entries as bit masks, from the rects
+// by a transpose.  8 keyframes in one view, both forward kernels, against two
+// warps per tile and a record gather by lane: 300 tiles 1200 -> 1052 us, 3072
+// tiles 467 -> 434; 24 keyframes x 24 views 12.5 -> 12.2 ms.
+template <int CHUNK>
+struct TailSmem {
+  static constexpr int W = CHUNK / 32;
+  float4 raw[CHUNK * REC_F4];
+  uint32_t rel[W][64];   // per pixel: the entries whose rect holds it
+  uint32_t bits[W][64];  // ... and those blended
+  FwdState st[64];
+  uint16_t list[W][CHUNK];
+  uint16_t apix[2][64];  // pixels still compositing, for this chunk and the next
+  int nact[2], next, item;
+};
+
+template <int CHUNK, bool DIST>
+__global__ void __launch_bounds__(CHUNK, 768 / CHUNK) k_render_tail(const RenderArgs A) {
+  constexpr int W = CHUNK / 32;
+  static_assert(W >= 2, "a thread per pixel");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  TailSmem<CHUNK>& S = *reinterpret_cast<TailSmem<CHUNK>*>(smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  const RastParams& P = A.P;
+  uint32_t n_eval = 0, n_blend = 0;
+  chain_release();
+  chain_wait();
+  // a failed binning (instance capacity exceeded) leaves no valid lists
+  if (A.hdr->status != 0) return;
+  const int n_items = (int)A.hdr->n_tails;
+  if (n_items == 0) return;
+  for (;;) {
+    __syncthreads();  // the last tile's state has been read
+    if (tid == 0) {
+      S.item = (int)atomicAdd(&A.hdr->queue_tail, 1u);
+      S.nact[0] = 0;
+    }
+    __syncthreads();
+    if (S.item >= n_items) break;
+    const uint2 from = __ldcg(A.tails + S.item);
+    const int t = (int)from.x;
+    const int v = find_view_by_tile(A.views, A.V, t);
+    const DView& vw = A.views[v];
+    const int lt = t - vw.tile_base;
+    const int tx0 = (lt % vw.tiles_x) * 8, ty0 = (lt / vw.tiles_x) * 8;
+    const int64_t HW = (int64_t)vw.W * vw.H;
+    const int ipx = tx0 + (tid & 7), ipy = ty0 + (tid >> 3);
+    const bool mine = tid < 64 && ipx < vw.W && ipy < vw.H;  // threads 0..63: a pixel each
+    const int64_t pix = vw.poff + (int64_t)ipy * vw.W + ipx;
+    const int64_t pix3 = 3 * vw.poff + (int64_t)ipy * vw.W + ipx;
+    const uint2 range = __ldg(A.ranges + t);
+    auto record_of = [&](int64_t i) -> uint32_t {  // of list entry i
+      if (i >= (int64_t)range.y) return 0xffffffffu;
+      const uint32_t sf = __ldg(A.vals + i);
+      if (!s2d_check((int64_t)sf >= vw.soff && (int64_t)sf < vw.soff + vw.scnt, A.hdr)) return 0xffffffffu;
+      return (uint32_t)(vw.rbase + ((int64_t)sf - vw.soff));
+    };
+    // the chunk's records, read one chunk ahead, and the next one's numbers
+    float4 f[REC_F4];
+    uint32_t ri = record_of((int64_t)from.y + tid);
+    bool ok = ri != 0xffffffffu;
+    load_records(A, ri, lane, f);
+    ri = record_of((int64_t)from.y + CHUNK + tid);
+    if (mine) {
+      const float T = __ldcg(A.tfinal + pix);
+      FwdState st = {fabsf(T), 0.f, 0.f, 0.f, __ldcg(A.dfinal + pix), 0.f, 0.f, 0.f, 0.f, __ldcg(A.last + pix), 0u};
+      if (A.rgb) {
+        st.C0 = __ldcg(A.rgb + pix3);
+        st.C1 = __ldcg(A.rgb + pix3 + HW);
+        st.C2 = __ldcg(A.rgb + pix3 + 2 * HW);
+      }
+      if (A.normal) {
+        st.N0 = __ldcg(A.normal + pix3);
+        st.N1 = __ldcg(A.normal + pix3 + HW);
+        st.N2 = __ldcg(A.normal + pix3 + 2 * HW);
+      }
+      if constexpr (DIST) st.Ds = __ldcg(A.dist + pix);
+      S.st[tid] = st;
+      if (__float_as_int(T) >= 0) S.apix[0][atomicAdd(&S.nact[0], 1)] = (uint16_t)tid;
+    }
+    for (int i = tid; i < W * 64; i += CHUNK) S.bits[0][i] = 0u;
+    __syncthreads();
+    int cur = 0;
+    for (int64_t base = from.y; base < range.y; base += CHUNK, cur ^= 1) {
+      const int n_act = S.nact[cur];
+      if (n_act == 0) break;
+      const int count = (int)min64(CHUNK, (int64_t)range.y - base);
+      // ---- stage: warp w has entries 32 w ... of the chunk
+      float4* raw = S.raw + wid * 32 * REC_F4;
+      store_records(A, base + 32 * wid, count - 32 * wid, lane, f, raw);
+      __syncwarp();
+      {
+        const float4 f4 = raw[lane * REC_F4 + 4];
+        const uint32_t r0 = __float_as_uint(f4.z), r1 = __float_as_uint(f4.w);
+        S.rel[wid][lane] = warp_transpose_bits(ok ? block_rect_mask(r0, r1, tx0, ty0) : 0u, lane);
+        S.rel[wid][32 + lane] = warp_transpose_bits(ok ? block_rect_mask(r0, r1, tx0, ty0 + 4) : 0u, lane);
+      }
+      if (tid == 0) {
+        S.nact[cur ^ 1] = 0;
+        S.next = 0;
+      }
+      ok = ri != 0xffffffffu;
+      load_records(A, ri, lane, f);
+      ri = record_of(base + 2 * CHUNK + tid);
+      __syncthreads();
+      // ---- the warps pull the pixels
+      for (;;) {
+        int k = 0;
+        if (lane == 0) k = atomicAdd(&S.next, 1);
+        k = __shfl_sync(0xffffffffu, k, 0);
+        if (k >= n_act) break;
+        const int pth = S.apix[cur][k];
+        // this pixel's entries of the chunk, ascending
+        int nrel = 0;
+#pragma unroll
+        for (int wd = 0; wd < W; wd++) {
+          const uint32_t bb = S.rel[wd][pth];
+          if ((bb >> lane) & 1u) S.list[wid][nrel + __popc(bb & lt_mask)] = (uint16_t)(wd * 32 + lane);
+          nrel += __popc(bb);
+        }
+        __syncwarp();
+        const float fx = (float)(tx0 + (pth & 7)) + 0.5f, fy = (float)(ty0 + (pth >> 3)) + 0.5f;
+        FwdState st = S.st[pth];
+        float acc[8] = {st.C0, st.C1, st.C2, st.D, st.N0, st.N1, st.N2, st.Ds};
+        float tt = st.T;
+        uint32_t lst = st.last;
+        bool dn = false;
+        for (int g = 0; g < nrel && !dn; g += 32) {
+          const bool has = g + lane < nrel;
+          const int j = has ? (int)S.list[wid][g + lane] : 0;
+          const float4* rec = S.raw + j * REC_F4;
+          const float4 f2 = rec[2], f3 = rec[3], f4 = rec[4];
+          Pair e;
+          float alpha = 0.f;
+          if (has) {
+            const float4 f0 = rec[0];
+            const float2 cl = unpack_half2_scaled(__float_as_uint(f0.z));
+            eval_pair(make_float4(f0.x, f0.y, cl.x, cl.y), rec[1], make_float4(f2.x, f2.y, f2.z, f0.w), fx, fy,
+                      P.lp_scale, P.alpha_max, e);
+            alpha = e.alpha;
+          }
+          const bool kept = has && alpha >= P.alpha_min;
+          const float om = kept ? __fsub_rn(1.f, alpha) : 1.f;
+          const float Pin = warp_scan_mul(om, lane);
+          float Pex = __shfl_up_sync(0xffffffffu, Pin, 1);
+          if (lane == 0) Pex = 1.f;
+          const float Tb = __fmul_rn(tt, Pex), Ta = __fmul_rn(tt, Pin);
+          const uint32_t stopb = __ballot_sync(0xffffffffu, kept && Ta < P.t_min);
+          const int sl = stopb ? __ffs(stopb) - 1 : 32;
+          const bool contrib = kept && lane < sl;
+          n_eval += (has && lane <= sl) ? 1u : 0u;
+          const uint32_t cb = __ballot_sync(0xffffffffu, contrib);
+          if (cb) {
+            const float w = contrib ? __fmul_rn(alpha, Tb) : 0.f;
+            float vals[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            float zpair = 0.f;
+            if (contrib) {
+              zpair = pair_depth(e, f4.y, f2.z, P.depth_ray);
+              vals[0] = w * f2.w; vals[1] = w * f3.x; vals[2] = w * f3.y;
+              vals[3] = w * zpair;
+              vals[4] = w * f3.z; vals[5] = w * f3.w; vals[6] = w * f4.x;
+            }
+            if constexpr (DIST) {
+              // depth sum in front of each pair: the pixel's so far, then the group's own terms before it
+              const float wz = vals[3];
+              const float Bb = acc[3] + (warp_scan_add(wz, lane) - wz);
+              vals[7] = contrib ? 2.f * w * (zpair * (1.f - Tb) - Bb) : 0.f;
+            }
+            warp_sum8_all(vals, lane);
+#pragma unroll
+            for (int q = 0; q < 8; q++) acc[q] += vals[q];
+            if (contrib) atomicOr(&S.bits[j >> 5][pth], 1u << (j & 31));
+            lst = (uint32_t)(base + __shfl_sync(0xffffffffu, j, 31 - __clz(cb)) + 1);
+          }
+          dn = stopb != 0u;
+          tt = dn ? __shfl_sync(0xffffffffu, Tb, sl) : __shfl_sync(0xffffffffu, Ta, 31);
+        }
+        if (lane == 0) {
+          S.st[pth] = FwdState{tt, acc[0], acc[1], acc[2], acc[3], acc[4], acc[5], acc[6], acc[7], lst, 0u};
+          if (!dn) S.apix[cur ^ 1][atomicAdd(&S.nact[cur ^ 1], 1)] = (uint16_t)pth;
+        }
+        __syncwarp();
+      }
+      __syncthreads();
+      // the blended masks, in the words of the tile's chunk
+      const int64_t word = (int64_t)(range.x >> 5) + t + ((base - (int64_t)range.x) >> 5);
+      const int nwd = (count + 31) >> 5;
+      const bool bm_ok = s2d_check(word + nwd <= A.bmask_words, A.hdr);
+      for (int i = tid; i < W * 64; i += CHUNK) {
+        const uint32_t b = S.bits[0][i];
+        S.bits[0][i] = 0u;
+        n_blend += __popc(b);
+        if (i < nwd * 64 && bm_ok) __stcs(A.bmask + word * 64 + i, b);
+      }
+    }
+    if (mine) {
+      const FwdState st = S.st[tid];
+      if (A.rgb) {
+        A.rgb[pix3] = __fmaf_rn(st.T, P.bg[0], st.C0);
+        A.rgb[pix3 + HW] = __fmaf_rn(st.T, P.bg[1], st.C1);
+        A.rgb[pix3 + 2 * HW] = __fmaf_rn(st.T, P.bg[2], st.C2);
+      }
+      if (A.depth) A.depth[pix] = st.D;
+      if (A.normal) {
+        A.normal[pix3] = st.N0;
+        A.normal[pix3 + HW] = st.N1;
+        A.normal[pix3 + 2 * HW] = st.N2;
+      }
+      if (A.alpha) A.alpha[pix] = 1.f - st.T;
+      if constexpr (DIST) A.dist[pix] = st.Ds;
+      A.tfinal[pix] = st.T;
+      A.last[pix] = st.last;
+      A.dfinal[pix] = st.D;
+    }
+  }
+  leave_queue(&A.hdr->queue_tail, &A.hdr->done_tail, &A.hdr->n_tails);
   if (P.stats) {
     unsigned long long a = n_eval, b = n_blend;
     for (int o = 16; o > 0; o >>= 1) {
@@ -1613,6 +1900,8 @@ static RenderArgs make_args(const Layout& L, const RastParams& P, char* ws, cons
   A.tfinal = reinterpret_cast<float*>(ws + L.tfinal);
   A.last = reinterpret_cast<uint32_t*>(ws + L.last);
   A.dfinal = reinterpret_cast<float*>(ws + L.dfinal);
+  A.chunk = 0;
+  A.tails = reinterpret_cast<uint2*>(ws + L.tile_class);  // the binning's lists, read no more
   A.rgb = A.depth = A.normal = A.alpha = A.dist = nullptr;
   A.d_rgb = A.d_depth = A.d_normal = A.d_alpha = A.d_dist = nullptr;
   return A;
@@ -1658,6 +1947,19 @@ static cudaError_t run_fwd_warp(const RenderArgs& A, cudaStream_t st) {
   static int64_t grid_T = -1;
   return run_warp_kernel<NP>(k_render_fwd_warp<NP, RAY, DIST>, sizeof(FwdWarpSmem<NP, RAY>) * WARPS, A, grid_T, grid,
                              st);
+}
+template <int CHUNK, bool DIST>
+static cudaError_t run_tail(const RenderArgs& A, cudaStream_t st) {
+  auto k = k_render_tail<CHUNK, DIST>;
+  constexpr size_t smem = sizeof(TailSmem<CHUNK>);
+  static int grid = -1;
+  static int64_t grid_T = -1;
+  if (grid < 0) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (grid < 0 || grid_T != A.T) {
+    grid = persistent_grid(k, CHUNK, smem, A.T);
+    grid_T = A.T;
+  }
+  return launch_chained(k, grid, CHUNK, smem, st, A);
 }
 template <int NP>
 static cudaError_t run_fwd_tiles8(const RenderArgs& A, cudaStream_t st) {
@@ -1726,8 +2028,16 @@ cudaError_t launch_render_fwd(const Layout& L, const RastParams& P, int chunk, c
   A.normal = normal;
   A.alpha = alpha;
   A.dist = dist;
-  if (P.tile_w == 8 && P.tile_h == 8)
-    return A.T > (int64_t)FW_WHOLE_TILES_PER_SM * sm_count() ? run_fwd_tiles8<2>(A, st) : run_fwd_tiles8<1>(A, st);
+  A.chunk = chunk;
+  if (P.tile_w == 8 && P.tile_h == 8) {
+    if (chunk != 64 && chunk != 128 && chunk != 256) return cudaErrorInvalidValue;
+    const cudaError_t e =
+        A.T > (int64_t)FW_WHOLE_TILES_PER_SM * sm_count() ? run_fwd_tiles8<2>(A, st) : run_fwd_tiles8<1>(A, st);
+    if (e != cudaSuccess) return e;
+    if (chunk == 64) return A.dist ? run_tail<64, true>(A, st) : run_tail<64, false>(A, st);
+    if (chunk == 128) return A.dist ? run_tail<128, true>(A, st) : run_tail<128, false>(A, st);
+    return A.dist ? run_tail<256, true>(A, st) : run_tail<256, false>(A, st);
+  }
   S2D_DISPATCH(run_fwd, P.tile_w, P.tile_h, chunk, A, st);
 }
 

@@ -53,8 +53,9 @@ struct Header {
   uint32_t queue_fwd, queue_bwd; // persistent work queues
   unsigned long long stat[8];    // pair counters, see STAT_*
   uint32_t queue_aux;            // work queue of the error-attribution pass
-  uint32_t done_fwd, done_bwd, done_aux;  // CTAs that have left each queue's kernel
-  uint32_t pad[28];
+  uint32_t done_fwd, done_bwd, done_aux, done_tail;  // CTAs that have left each queue's kernel
+  uint32_t n_tails, queue_tail;  // 8x8 tiles handed over by the forward: their number, their work queue
+  uint32_t pad[25];
 };
 static_assert(sizeof(Header) <= 256, "Header layout");
 enum { STAT_FWD_EVAL = 0, STAT_FWD_BLEND = 1, STAT_BWD_EVAL = 2, STAT_BWD_BLEND = 3, STAT_BWD_OUTSIDE = 4 };
@@ -248,14 +249,15 @@ __device__ __forceinline__ float2 unpack_half2_scaled(uint32_t u) {
   return make_float2(f.x * (1.0f / 65536.0f), f.y * (1.0f / 65536.0f));
 }
 
-// Leaves a persistent kernel's work queue: the last CTA to leave sets it (and
-// the count of those that left) back to zero for the kernel's next launch.
-// Every thread calls it, once, after the CTA's last item.
-__device__ __forceinline__ void leave_queue(uint32_t* queue, uint32_t* done) {
+// Leaves a persistent kernel's work queue: the last CTA to leave sets it, the
+// count of those that left and `more` back to zero for the kernel's next
+// launch.  Every thread calls it, once, after the CTA's last item.
+__device__ __forceinline__ void leave_queue(uint32_t* queue, uint32_t* done, uint32_t* more = nullptr) {
   __syncthreads();
   if (threadIdx.x == 0 && atomicAdd(done, 1u) == gridDim.x - 1) {
     *queue = 0u;
     *done = 0u;
+    if (more) *more = 0u;
   }
 }
 
