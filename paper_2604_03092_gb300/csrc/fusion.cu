@@ -5,9 +5,10 @@
 // The accumulation map is the forward's alpha output A = 1 - T_final at the
 // new keyframe's pose; the frame's new primitives are per pixel, so the gate
 // is an ordered stream compaction: keep_idx lists, in ascending order, the
-// pixels with A < tau.  Three launches: per-block counts, one block scanning
-// the counts (which also writes the total), and a scatter in which each
-// block ranks its kept pixels with warp ballots.
+// pixels with A < tau.  Two chained launches: per-block counts, and a scatter
+// in which each block adds up the counts before its own and ranks its kept
+// pixels with warp ballots.  (Far too many blocks for that take a scan of the
+// counts in between.)
 #include <cuda_runtime.h>
 
 #include "splat2d_internal.cuh"
@@ -22,8 +23,25 @@ __device__ __forceinline__ bool gate_keep(const float* alpha, int64_t i, int64_t
   return i < n && alpha[i] < tau;  // false for NaN
 }
 
+// Up to this many blocks, each adds up the counts before its own (at most 16
+// loads a thread, under the scatter's own loads); a scan of them by one block
+// in a launch of its own is 2.9 us for 200 or 300 blocks.
+constexpr int64_t SUM_BLOCKS = 4096;
+
+// The counts before this block's: its thread's part of them, or all of them
+// (thread 0) where they have been scanned.
+template <int THREADS>
+__device__ __forceinline__ uint32_t counts_before(const uint32_t* __restrict__ count, bool scanned) {
+  if (scanned) return threadIdx.x == 0 ? count[blockIdx.x] : 0u;
+  uint32_t c = 0;
+  for (uint32_t i = threadIdx.x; i < blockIdx.x; i += THREADS) c += count[i];
+  return c;
+}
+
 __global__ void __launch_bounds__(GATE_THREADS) k_gate_count(const float* __restrict__ alpha, int64_t n, float tau,
                                                              uint32_t* __restrict__ block_count) {
+  chain_release();
+  chain_wait();
   __shared__ uint32_t s_w[GATE_THREADS / 32];
   const int64_t base = (int64_t)blockIdx.x * GATE_TILE;
   uint32_t c = 0;
@@ -42,6 +60,8 @@ __global__ void __launch_bounds__(GATE_THREADS) k_gate_count(const float* __rest
 // One block: exclusive scan of the block counts in place; the total goes to *n_keep.
 __global__ void __launch_bounds__(1024) k_gate_scan(uint32_t* __restrict__ block_count, int64_t nb,
                                                     int64_t* __restrict__ n_keep) {
+  chain_release();
+  chain_wait();
   __shared__ unsigned long long s_w[32];
   __shared__ unsigned long long s_carry;
   if (threadIdx.x == 0) s_carry = 0;
@@ -76,32 +96,46 @@ __global__ void __launch_bounds__(1024) k_gate_scan(uint32_t* __restrict__ block
 }
 
 __global__ void __launch_bounds__(GATE_THREADS) k_gate_scatter(const float* __restrict__ alpha, int64_t n, float tau,
-                                                               const uint32_t* __restrict__ block_offset,
-                                                               uint32_t* __restrict__ keep_idx) {
-  __shared__ uint32_t s_w[GATE_THREADS / 32];
-  __shared__ uint32_t s_run;
+                                                               const uint32_t* __restrict__ count, bool scanned,
+                                                               uint32_t* __restrict__ keep_idx,
+                                                               int64_t* __restrict__ n_keep) {
+  constexpr int NW = GATE_THREADS / 32;
+  static_assert(GATE_PER_THREAD * NW == 32, "a lane per (round, warp)");
+  __shared__ uint32_t s_kept[32], s_before[NW];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint32_t lt = (1u << lane) - 1u;
   const int64_t base = (int64_t)blockIdx.x * GATE_TILE;
-  if (threadIdx.x == 0) s_run = block_offset[blockIdx.x];
-  __syncthreads();
+  chain_release();
+  chain_wait();
   // rounds of GATE_THREADS consecutive pixels keep the output in ascending order
+  uint32_t m[GATE_PER_THREAD];
+#pragma unroll
+  for (int k = 0; k < GATE_PER_THREAD; k++)
+    m[k] = gate_keep(alpha, base + k * GATE_THREADS + threadIdx.x, n, tau) ? 1u : 0u;
+  const uint32_t part = __reduce_add_sync(0xffffffffu, counts_before<GATE_THREADS>(count, scanned));
+  if (lane == 0) s_before[wid] = part;
+#pragma unroll
   for (int k = 0; k < GATE_PER_THREAD; k++) {
-    const int64_t i = base + k * GATE_THREADS + threadIdx.x;
-    const bool keep = gate_keep(alpha, i, n, tau);
-    const uint32_t m = __ballot_sync(0xffffffffu, keep);
-    if (lane == 0) s_w[wid] = __popc(m);
-    __syncthreads();
-    uint32_t before = s_run;
-    for (int w = 0; w < wid; w++) before += s_w[w];
-    if (keep) keep_idx[before + __popc(m & lt)] = (uint32_t)i;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t t = 0;
-      for (int w = 0; w < GATE_THREADS / 32; w++) t += s_w[w];
-      s_run += t;
-    }
-    __syncthreads();
+    m[k] = __ballot_sync(0xffffffffu, m[k]);
+    if (lane == 0) s_kept[k * NW + wid] = __popc(m[k]);
+  }
+  __syncthreads();
+  uint32_t start = 0;
+#pragma unroll
+  for (int w = 0; w < NW; w++) start += s_before[w];
+  const uint32_t c = s_kept[lane];
+  uint32_t x = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (!scanned && blockIdx.x == gridDim.x - 1 && threadIdx.x == GATE_THREADS - 1) *n_keep = (int64_t)start + x;
+#pragma unroll
+  for (int k = 0; k < GATE_PER_THREAD; k++) {
+    const uint32_t before = start + __shfl_sync(0xffffffffu, x - c, k * NW + wid);
+    if ((m[k] >> lane) & 1u)
+      keep_idx[before + __popc(m[k] & lt)] = (uint32_t)(base + k * GATE_THREADS + threadIdx.x);
   }
 }
 
@@ -115,13 +149,12 @@ cudaError_t launch_accum_gate(const float* alpha, int64_t n, float tau, uint32_t
   const int64_t nb = (n + GATE_TILE - 1) / GATE_TILE;
   if (nb == 0) return cudaMemsetAsync(n_keep, 0, sizeof(int64_t), st);
   uint32_t* counts = static_cast<uint32_t*>(tmp);
-  k_gate_count<<<(unsigned)nb, GATE_THREADS, 0, st>>>(alpha, n, tau, counts);
-  count_launches(1);
-  k_gate_scan<<<1, 1024, 0, st>>>(counts, nb, n_keep);
-  count_launches(1);
-  k_gate_scatter<<<(unsigned)nb, GATE_THREADS, 0, st>>>(alpha, n, tau, counts, keep_idx);
-  count_launches(1);
-  return cudaGetLastError();
+  cudaError_t e = launch_chained(k_gate_count, (int)nb, GATE_THREADS, 0, st, alpha, n, tau, counts);
+  if (e != cudaSuccess) return e;
+  const bool scanned = nb > SUM_BLOCKS;
+  if (scanned && (e = launch_chained(k_gate_scan, 1, 1024, 0, st, counts, nb, n_keep)) != cudaSuccess) return e;
+  return launch_chained(k_gate_scatter, (int)nb, GATE_THREADS, 0, st, alpha, n, tau, counts, scanned, keep_idx,
+                        n_keep);
 }
 
 // ---------------------------------------------------------------------------
@@ -133,8 +166,8 @@ cudaError_t launch_accum_gate(const float* alpha, int64_t n, float tau, uint32_t
 // block's depth variation (largest minus smallest camera-frame depth of its
 // primitives) exceeds tau_d, in which case its primitives are kept.  Output
 // is ordered: blocks in row-major order, a kept block's primitives in
-// row-major order.  One thread per block; the same count / scan / scatter
-// scheme as the gate.
+// row-major order.  One thread per block; the same count and scatter scheme
+// as the gate.
 // ---------------------------------------------------------------------------
 constexpr int VOX_THREADS = 256;
 
@@ -150,34 +183,47 @@ struct VoxOut {
   int32_t* block;
 };
 
-// Members of block b (row-major) and whether it merges.
-__device__ __forceinline__ int vox_members(const VoxIn& I, int64_t b, int64_t (&idx)[4], bool& merge) {
-  const int bx = (int)(b % I.bw), by = (int)(b / I.bw);
-  int n = 0;
-  for (int dy = 0; dy < 2; dy++)
-    for (int dx = 0; dx < 2; dx++) {
-      const int x = 2 * bx + dx, y = 2 * by + dy;
-      if (x < I.W && y < I.H) idx[n++] = (int64_t)y * I.W + x;
+// The four places of block b (row-major): their indices, which of them lie in
+// the image (the others' index is the first one's), and whether the block
+// merges.
+struct VoxBlock {
+  int64_t idx[4];
+  bool in[4];
+  int n;
+  __device__ __forceinline__ VoxBlock(const VoxIn& I, int64_t b) {
+    const int x = 2 * (int)(b % I.bw), y = 2 * (int)(b / I.bw);
+    const int64_t first = (int64_t)y * I.W + x;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      in[k] = x + (k & 1) < I.W && y + (k >> 1) < I.H;
+      idx[k] = in[k] ? first + (k & 1) + (int64_t)(k >> 1) * I.W : first;
     }
-  float zmin = I.means[3 * idx[0] + 2], zmax = zmin;
-  for (int k = 1; k < n; k++) {
-    const float z = I.means[3 * idx[k] + 2];
-    zmin = fminf(zmin, z);
-    zmax = fmaxf(zmax, z);
+    n = 1 + in[1] + in[2] + in[3];
   }
-  merge = !(zmax - zmin > I.tau_d);
-  return n;
-}
+  __device__ __forceinline__ bool merges(const float (&z)[4], float tau_d) const {
+    float zmin = z[0], zmax = z[0];
+#pragma unroll
+    for (int k = 1; k < 4; k++)
+      if (in[k]) {
+        zmin = fminf(zmin, z[k]);
+        zmax = fmaxf(zmax, z[k]);
+      }
+    return !(zmax - zmin > tau_d);
+  }
+};
 
 __global__ void __launch_bounds__(VOX_THREADS) k_vox_count(const VoxIn I, uint32_t* __restrict__ block_count) {
   __shared__ uint32_t s_w[VOX_THREADS / 32];
   const int64_t b = (int64_t)blockIdx.x * VOX_THREADS + threadIdx.x;
+  chain_release();
+  chain_wait();
   uint32_t c = 0;
   if (b < I.nb) {
-    int64_t idx[4];
-    bool merge;
-    const int n = vox_members(I, b, idx, merge);
-    c = merge ? 1u : (uint32_t)n;
+    const VoxBlock B(I, b);
+    float z[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) z[k] = I.means[3 * B.idx[k] + 2];
+    c = B.merges(z, I.tau_d) ? 1u : (uint32_t)B.n;
   }
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = c;
@@ -189,61 +235,103 @@ __global__ void __launch_bounds__(VOX_THREADS) k_vox_count(const VoxIn I, uint32
   }
 }
 
-__device__ __forceinline__ void vox_copy(const VoxIn& I, const VoxOut& O, int64_t i, int64_t o, int32_t b) {
-  for (int k = 0; k < 3; k++) O.means[3 * o + k] = I.means[3 * i + k];
-  for (int k = 0; k < 2; k++) O.scales[2 * o + k] = I.scales[2 * i + k];
-  for (int k = 0; k < 4; k++) O.quats[4 * o + k] = I.quats[4 * i + k];
-  O.opacity[o] = I.opacity[i];
-  for (int k = 0; k < 3; k++) O.rgb[3 * o + k] = I.rgb[3 * i + k];
-  if (O.block) O.block[o] = b;
-}
-
-__global__ void __launch_bounds__(VOX_THREADS) k_vox_scatter(const VoxIn I, const uint32_t* __restrict__ block_offset,
-                                                             const VoxOut O) {
-  __shared__ uint32_t s_w[VOX_THREADS / 32];
+// Latency-bound (some 320 blocks per SM for a 512x384 keyframe): all 52 floats
+// of a block's primitives are read at once, before its place is known.  With a
+// loop over the members behind the scan, and the scan of the counts in a launch
+// of its own, such a keyframe took 4.1 + 2.8 + 13.6 us (count, scan, scatter);
+// now 3.4 + 8.4 us.
+__global__ void __launch_bounds__(VOX_THREADS) k_vox_scatter(const VoxIn I, const uint32_t* __restrict__ count,
+                                                             bool scanned, const VoxOut O,
+                                                             int64_t* __restrict__ n_out) {
+  constexpr int NW = VOX_THREADS / 32;
+  __shared__ uint32_t s_w[NW], s_before[NW];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t b = (int64_t)blockIdx.x * VOX_THREADS + threadIdx.x;
-  int64_t idx[4] = {0, 0, 0, 0};
-  bool merge = true;
-  int n = 0;
-  if (b < I.nb) n = vox_members(I, b, idx, merge);
-  const uint32_t c = b < I.nb ? (merge ? 1u : (uint32_t)n) : 0u;
+  chain_release();
+  chain_wait();
+  const VoxBlock B(I, b < I.nb ? b : 0);
+  float mu[4][3], sc[4][2], q[4][4], op[4], rgb[4][3];
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    const int64_t i = B.idx[k];
+#pragma unroll
+    for (int j = 0; j < 3; j++) mu[k][j] = I.means[3 * i + j];
+#pragma unroll
+    for (int j = 0; j < 2; j++) sc[k][j] = I.scales[2 * i + j];
+#pragma unroll
+    for (int j = 0; j < 4; j++) q[k][j] = I.quats[4 * i + j];
+    op[k] = I.opacity[i];
+#pragma unroll
+    for (int j = 0; j < 3; j++) rgb[k][j] = I.rgb[3 * i + j];
+  }
+  const uint32_t part = __reduce_add_sync(0xffffffffu, counts_before<VOX_THREADS>(count, scanned));
+  const float z[4] = {mu[0][2], mu[1][2], mu[2][2], mu[3][2]};
+  const bool merge = B.merges(z, I.tau_d);
+  const uint32_t c = b < I.nb ? (merge ? 1u : (uint32_t)B.n) : 0u;
   uint32_t x = c;
+#pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
-  if (lane == 31) s_w[wid] = x;
+  if (lane == 31) {
+    s_w[wid] = x;
+    s_before[wid] = part;
+  }
   __syncthreads();
-  uint32_t before = block_offset[blockIdx.x];
-  for (int w = 0; w < wid; w++) before += s_w[w];
-  const int64_t o = (int64_t)before + (x - c);
+  uint32_t before = 0;
+#pragma unroll
+  for (int w = 0; w < NW; w++) before += s_before[w] + (w < wid ? s_w[w] : 0u);
+  if (!scanned && blockIdx.x == gridDim.x - 1 && threadIdx.x == VOX_THREADS - 1) *n_out = (int64_t)before + x;
   if (b >= I.nb) return;
+  int64_t o = (int64_t)before + (x - c);
+  auto put = [&](const float (&m)[3], const float (&s2)[2], const float (&r)[4], float a, const float (&col)[3]) {
+#pragma unroll
+    for (int j = 0; j < 3; j++) O.means[3 * o + j] = m[j];
+#pragma unroll
+    for (int j = 0; j < 2; j++) O.scales[2 * o + j] = s2[j];
+#pragma unroll
+    for (int j = 0; j < 4; j++) O.quats[4 * o + j] = r[j];
+    O.opacity[o] = a;
+#pragma unroll
+    for (int j = 0; j < 3; j++) O.rgb[3 * o + j] = col[j];
+    if (O.block) O.block[o] = (int32_t)b;
+    o++;
+  };
   if (!merge) {
-    for (int k = 0; k < n; k++) vox_copy(I, O, idx[k], o + k, (int32_t)b);
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+      if (B.in[k]) put(mu[k], sc[k], q[k], op[k], rgb[k]);
     return;
   }
-  const float inv = 1.0f / (float)n;
-  float m[3] = {0.f, 0.f, 0.f}, sc[2] = {0.f, 0.f}, q[4] = {0.f, 0.f, 0.f, 0.f}, op = 0.f, c3[3] = {0.f, 0.f, 0.f};
-  const float* q1 = I.quats + 4 * idx[0];
-  for (int k = 0; k < n; k++) {
-    const int64_t i = idx[k];
-    for (int j = 0; j < 3; j++) m[j] += I.means[3 * i + j];
-    for (int j = 0; j < 2; j++) sc[j] += I.scales[2 * i + j];
-    const float* qi = I.quats + 4 * i;
-    const float d = qi[0] * q1[0] + qi[1] * q1[1] + qi[2] * q1[2] + qi[3] * q1[3];
+  const float inv = 1.0f / (float)B.n;
+  float m[3] = {0.f, 0.f, 0.f}, s2[2] = {0.f, 0.f}, r[4] = {0.f, 0.f, 0.f, 0.f}, a = 0.f, col[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    if (!B.in[k]) continue;
+#pragma unroll
+    for (int j = 0; j < 3; j++) m[j] += mu[k][j];
+#pragma unroll
+    for (int j = 0; j < 2; j++) s2[j] += sc[k][j];
+    const float d = q[k][0] * q[0][0] + q[k][1] * q[0][1] + q[k][2] * q[0][2] + q[k][3] * q[0][3];
     const float sg = d >= 0.f ? 1.f : -1.f;  // align to the block's first quaternion
-    for (int j = 0; j < 4; j++) q[j] += sg * qi[j];
-    op += I.opacity[i];
-    for (int j = 0; j < 3; j++) c3[j] += I.rgb[3 * i + j];
+#pragma unroll
+    for (int j = 0; j < 4; j++) r[j] += sg * q[k][j];
+    a += op[k];
+#pragma unroll
+    for (int j = 0; j < 3; j++) col[j] += rgb[k][j];
   }
-  const float qn = sqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
-  for (int j = 0; j < 3; j++) O.means[3 * o + j] = m[j] * inv;
-  for (int j = 0; j < 2; j++) O.scales[2 * o + j] = sc[j] * inv;
-  for (int j = 0; j < 4; j++) O.quats[4 * o + j] = q[j] / qn;
-  O.opacity[o] = op * inv;
-  for (int j = 0; j < 3; j++) O.rgb[3 * o + j] = c3[j] * inv;
-  if (O.block) O.block[o] = (int32_t)b;
+  const float qn = sqrtf(r[0] * r[0] + r[1] * r[1] + r[2] * r[2] + r[3] * r[3]);
+#pragma unroll
+  for (int j = 0; j < 3; j++) {
+    m[j] *= inv;
+    col[j] *= inv;
+  }
+#pragma unroll
+  for (int j = 0; j < 2; j++) s2[j] *= inv;
+#pragma unroll
+  for (int j = 0; j < 4; j++) r[j] /= qn;
+  put(m, s2, r, a * inv, col);
 }
 
 size_t voxelize_tmp_size(int32_t W, int32_t H) {
@@ -266,13 +354,11 @@ cudaError_t launch_voxelize(const splat2d_surfels& in, int32_t W, int32_t H, flo
   if (I.nb == 0) return cudaMemsetAsync(n_out, 0, sizeof(int64_t), st);
   const int64_t g = (I.nb + VOX_THREADS - 1) / VOX_THREADS;
   uint32_t* counts = static_cast<uint32_t*>(tmp);
-  k_vox_count<<<(unsigned)g, VOX_THREADS, 0, st>>>(I, counts);
-  count_launches(1);
-  k_gate_scan<<<1, 1024, 0, st>>>(counts, g, n_out);
-  count_launches(1);
-  k_vox_scatter<<<(unsigned)g, VOX_THREADS, 0, st>>>(I, counts, O);
-  count_launches(1);
-  return cudaGetLastError();
+  cudaError_t e = launch_chained(k_vox_count, (int)g, VOX_THREADS, 0, st, I, counts);
+  if (e != cudaSuccess) return e;
+  const bool scanned = g > SUM_BLOCKS;
+  if (scanned && (e = launch_chained(k_gate_scan, 1, 1024, 0, st, counts, g, n_out)) != cudaSuccess) return e;
+  return launch_chained(k_vox_scatter, (int)g, VOX_THREADS, 0, st, I, counts, scanned, O, n_out);
 }
 
 // ---------------------------------------------------------------------------
