@@ -906,8 +906,11 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
         }
       }
       if (!any_bits<NP>(live_px)) {
-        if (NP == 1) continue;  // up to the next chunk, for the other half
-        break;
+        if (NP == 2) break;
+        // up to the next chunk, with the other half: it may go on blending, and
+        // the words it writes are then read for all of the tile's pixels
+        if (s2d_check((int64_t)word < A.bmask_words, A.hdr)) __stcs(A.bmask + (size_t)word * 64 + 32 * half + lane, 0u);
+        continue;
       }
       const int count = (int)min64(32, (int64_t)range.y - base);
       const uint32_t sf = ent;
