@@ -192,7 +192,7 @@ bool compute_layout(const splat2d_config* cfg, const splat2d_problem* prob, Layo
 }
 
 static RastParams make_params(const splat2d_config* c) {
-  RastParams P;
+  RastParams P = {};
   P.alpha_min = c->alpha_min;
   P.alpha_max = c->alpha_max;
   P.t_min = c->t_min;
@@ -202,6 +202,8 @@ static RastParams make_params(const splat2d_config* c) {
   P.bg[0] = c->bg[0]; P.bg[1] = c->bg[1]; P.bg[2] = c->bg[2];
   P.tile_w = c->tile_w;
   P.tile_h = c->tile_h;
+  while (1 << P.tile_w_log2 < P.tile_w) P.tile_w_log2++;
+  while (1 << P.tile_h_log2 < P.tile_h) P.tile_h_log2++;
   P.stats = (c->flags & SPLAT2D_FLAG_NO_STATS) ? 0 : 1;
   P.depth_ray = (c->flags & SPLAT2D_FLAG_DEPTH_RAY) ? 1 : 0;
   const int tail = (int)((c->flags >> SPLAT2D_FLAG_TAIL_SHIFT) & 0xffu);

@@ -40,7 +40,7 @@ struct TileBinArgs {
   const DView* views;
   int32_t V;
   int64_t R;
-  int32_t tile_w, tile_h;
+  int32_t tile_w_log2, tile_h_log2;
   uint32_t* counts;   // per tile: instances (count pass) / next free bucket slot (scatter, from the scan)
   unsigned long long* bucket;
   int64_t cap;        // instance capacity (bucket length)
@@ -167,8 +167,8 @@ __global__ void __launch_bounds__(256) k_tile_bin(const TileBinArgs A) {
       while (v + 1 < A.V && __ldg(&A.views[v + 1].rbase) <= r) v++;
       const DView& vw = A.views[v];
       const uint32_t q0 = e.y, q1 = e.z;
-      const int tx0 = (int)(q0 & 0xffffu) / A.tile_w, ty0 = (int)(q0 >> 16) / A.tile_h;
-      w = (int)(q1 & 0xffffu) / A.tile_w - tx0 + 1;
+      const int tx0 = (int)(q0 & 0xffffu) >> A.tile_w_log2, ty0 = (int)(q0 >> 16) >> A.tile_h_log2;
+      w = ((int)(q1 & 0xffffu) >> A.tile_w_log2) - tx0 + 1;
       t = (uint32_t)(vw.tile_base + ty0 * vw.tiles_x + tx0);
       wrap = (uint32_t)(vw.tiles_x - w + 1);
       left = w;
@@ -1043,8 +1043,8 @@ cudaError_t launch_bin_tiles(const Layout& L, const RastParams& P, char* ws, cud
   A.views = reinterpret_cast<const DView*>(ws + L.views);
   A.V = L.V;
   A.R = L.R;
-  A.tile_w = P.tile_w;
-  A.tile_h = P.tile_h;
+  A.tile_w_log2 = P.tile_w_log2;
+  A.tile_h_log2 = P.tile_h_log2;
   A.counts = counts;
   A.bucket = reinterpret_cast<unsigned long long*>(ws + L.keys1);
   A.cap = L.cap;

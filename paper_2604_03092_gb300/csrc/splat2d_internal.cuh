@@ -123,6 +123,7 @@ struct RastParams {
   float lp_r;       // sigma_lp (pixels) for the extent
   float bg[3];
   int32_t tile_w, tile_h;
+  int32_t tile_w_log2, tile_h_log2;  // the sizes are powers of two
   int32_t stats;    // keep pair counters
   int32_t fwd_tail; // forward: share the tile's pixels across warps below this many active per warp
   int32_t depth_ray; // depth output from the ray-splat intersection (SPLAT2D_FLAG_DEPTH_RAY)
