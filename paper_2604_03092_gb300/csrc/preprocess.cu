@@ -84,14 +84,17 @@ struct Surfel {
   bool valid;
 };
 
-__device__ __forceinline__ void load_surfel(const splat2d_surfels& S, int64_t s, Surfel& f) {
+// Center, scales and opacity; the rotation separately.
+__device__ __forceinline__ void load_extent(const splat2d_surfels& S, int64_t s, Surfel& f) {
   f.mx = __ldg(S.means + 3 * s + 0);
   f.my = __ldg(S.means + 3 * s + 1);
   f.mz = __ldg(S.means + 3 * s + 2);
   f.su = __ldg(S.scales + 2 * s + 0);
   f.sv = __ldg(S.scales + 2 * s + 1);
-  float4 q = __ldg(reinterpret_cast<const float4*>(S.quats) + s);
   f.op = __ldg(S.opacity + s);
+}
+__device__ __forceinline__ void load_rotation(const splat2d_surfels& S, int64_t s, Surfel& f) {
+  float4 q = __ldg(reinterpret_cast<const float4*>(S.quats) + s);
   float n2 = q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w;
   f.valid = n2 > 0.f && isfinite(n2);
   f.qn = sqrtf(n2);
@@ -161,6 +164,33 @@ struct PreArgs {
   float4* rgrad;
   Header* hdr;
 };
+
+// Whether project_one would find no pixel, from the center and the longest
+// axis alone: the sphere around the extent, widened by 1% and by the rounding
+// of the center, lies nearer than z_near, or beyond one side of the image by two
+// pixels more than the low-pass extent.  Beyond a side only where the center
+// is more than two radii deep, so the projected ellipse is small against its
+// distance and its computed extents are good to far less than these pixels.
+// False for any NaN.
+__device__ __forceinline__ bool surely_outside(const DView& vw, const RastParams& P, const Surfel& f) {
+  float rr = 0.f;  // Frobenius norm of R squared: it bounds R's stretch, whatever R is
+#pragma unroll
+  for (int k = 0; k < 9; k++) rr = fmaf(vw.R[k], vw.R[k], rr);
+  const float x = fmaf(vw.R[0], f.mx, fmaf(vw.R[1], f.my, fmaf(vw.R[2], f.mz, vw.t[0])));
+  const float y = fmaf(vw.R[3], f.mx, fmaf(vw.R[4], f.my, fmaf(vw.R[5], f.mz, vw.t[1])));
+  const float z = fmaf(vw.R[6], f.mx, fmaf(vw.R[7], f.my, fmaf(vw.R[8], f.mz, vw.t[2])));
+  const float far = fabsf(f.mx) + fabsf(f.my) + fabsf(f.mz);
+  const float rad = fmaf(sqrtf(rr), fmaf(1.01f * f.kk, fmaxf(fabsf(f.su), fabsf(f.sv)), 1e-5f * far),
+                         1e-5f * (fabsf(vw.t[0]) + fabsf(vw.t[1]) + fabsf(vw.t[2])));
+  if (z + rad < P.z_near) return true;
+  if (!(z > 2.f * rad)) return false;
+  // the side px = b, b = left or right bound: fx x - (b - cx) z, over the norm of (fx, b - cx) or more
+  const float m = fmaf(P.lp_r, f.kk, 2.f);
+  const float l = vw.cx + m, r = (float)vw.W + m - vw.cx, u = vw.cy + m, d = (float)vw.H + m - vw.cy;
+  const float ax = fabsf(vw.fx), ay = fabsf(vw.fy), px = vw.fx * x, py = vw.fy * y;
+  return -fmaf(l, z, px) > rad * (ax + fabsf(l)) || fmaf(-r, z, px) > rad * (ax + fabsf(r)) ||
+         -fmaf(u, z, py) > rad * (ay + fabsf(u)) || fmaf(-d, z, py) > rad * (ay + fabsf(d));
+}
 
 __device__ __forceinline__ uint32_t project_one(const PreArgs& A, const DView& vw, const Surfel& f,
                                                 float4* rec_out) {
@@ -273,6 +303,12 @@ __device__ __forceinline__ uint32_t project_one(const PreArgs& A, const DView& v
 // run time only, and colours read where the surfel is visible: 48 keyframes in
 // one view 226 -> 189 us, 8 keyframes x 8 views 330 -> 308 (binning 852 ->
 // 840), 24 x 24 2395 -> 2221 (5861 -> 5784).
+// ONE_VIEW: no surfel is in two views.  Most of a map is then outside its
+// view, and the others are told from center and size, before the rotation is
+// read: 48 keyframes in one view 187 -> 154 us.  With more views a surfel most
+// are inside, and the test costs more than it saves: 8 keyframes x 8 views 308
+// -> 361, 24 x 24 2222 -> 2515.
+template <bool ONE_VIEW>
 __global__ void __launch_bounds__(256, 3) k_preprocess(const PreArgs A) {
   chain_release();
   chain_wait();
@@ -283,13 +319,22 @@ __global__ void __launch_bounds__(256, 3) k_preprocess(const PreArgs A) {
     const DGroup grp = A.groups[g];
     const int64_t s = grp.soff + (w - grp.wbase);
     Surfel f;
-    load_surfel(A.S, s, f);
+    load_extent(A.S, s, f);
+    if (!ONE_VIEW) load_rotation(A.S, s, f);
     // the extent's k^2 = 2 ln(op / alpha_min): the surfel's, whatever the view
     f.k2 = 2.0f * logf(f.op / A.P.alpha_min);
     f.kk = sqrtf(f.k2);
     for (int v = grp.v0; v < grp.v1; v++) {
       const DView& vw = A.views[v];
       const int64_t rec = vw.rbase + (s - vw.soff);
+      if (ONE_VIEW) {
+        if (surely_outside(vw, A.P, f)) {
+          A.ntiles[rec] = 0u;
+          A.bins[rec] = make_uint4(0u, 0u, 0u, 0u);
+          continue;
+        }
+        load_rotation(A.S, s, f);
+      }
       float4 r[REC_F4];
       uint32_t nt = project_one(A, vw, f, r);
       A.ntiles[rec] = nt;
@@ -330,7 +375,8 @@ cudaError_t launch_preprocess(const splat2d_surfels* S, const Layout& L, const R
   int64_t blocks = (n_work + 255) / 256;
   int64_t cap = (int64_t)sm_count() * 16;
   if (blocks > cap) blocks = cap;
-  return launch_chained(k_preprocess, (int)blocks, 256, 0, st, A);
+  const bool one_view = L.V == L.G && !L.groups_overlap;
+  return launch_chained(one_view ? k_preprocess<true> : k_preprocess<false>, (int)blocks, 256, 0, st, A);
 }
 
 // ---------------------------------------------------------------------------
@@ -376,7 +422,10 @@ __global__ void __launch_bounds__(256, 4) k_preprocess_bwd(const PreBwdArgs A) {
     const DGroup grp = A.groups[g];
     const int64_t s = live ? grp.soff + (w - grp.wbase) : 0;
     Surfel f;
-    if (live) load_surfel(A.S, s, f);
+    if (live) {
+      load_extent(A.S, s, f);
+      load_rotation(A.S, s, f);
+    }
     // world-frame accumulators over the views of this surfel
     float gm[3] = {0.f, 0.f, 0.f}, gsu = 0.f, gsv = 0.f, gop = 0.f, gc[3] = {0.f, 0.f, 0.f};
     float gtu[3] = {0.f, 0.f, 0.f}, gtv[3] = {0.f, 0.f, 0.f}, gnw[3] = {0.f, 0.f, 0.f};
