@@ -399,7 +399,14 @@ struct PreBwdArgs {
 
 constexpr int kPoseSlots = 64;  // per-block pose accumulators (views)
 
-__global__ void __launch_bounds__(256, 4) k_preprocess_bwd(const PreBwdArgs A) {
+// Bound by the latency of the gradient records and by issue.  A record that no
+// pixel touched, its gradient zero, adds nothing and skips the chain rule, a
+// warp of them the pose sums too.  Three CTAs per SM of 80 registers, for four
+// of 64 that spill; up to 24 blocks per SM, for 8, which left the last ones
+// uneven: one keyframe x 8 views 107 -> 92 us, 8 x 8 558 -> 486, 24 x 24 3481
+// -> 3141, 12 uneven submaps 440 -> 417 (48 blocks 94, 492, 3129, 420, without
+// the skip 92, 492, 3157, 422; each block adds its pose sums in FP32).
+__global__ void __launch_bounds__(256, 3) k_preprocess_bwd(const PreBwdArgs A) {
   __shared__ float s_pose[kPoseSlots][6];
   __shared__ int s_vfirst;
   chain_release();
@@ -437,6 +444,7 @@ __global__ void __launch_bounds__(256, 4) k_preprocess_bwd(const PreBwdArgs A) {
     for (int k = 0; k < nv_max; k++) {
       const int v = (k < nv) ? grp.v0 + k : -1;
       float pose[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      bool touched = false;
       if (v >= 0) {
         const DView& vw = A.views[v];
         const int64_t rec = vw.rbase + (s - vw.soff);
@@ -444,89 +452,90 @@ __global__ void __launch_bounds__(256, 4) k_preprocess_bwd(const PreBwdArgs A) {
           float4* gp = A.rgrad + rec * (GRAD_F / 4);
           const float4 q0 = gp[0], q1 = gp[1], q2 = gp[2], q3 = gp[3], q4 = gp[4];
           // leave the gradient record zero for the next reverse pass
-          const bool touched = (q0.x != 0.f) | (q0.y != 0.f) | (q0.z != 0.f) | (q0.w != 0.f) | (q1.x != 0.f) |
+          touched = (q0.x != 0.f) | (q0.y != 0.f) | (q0.z != 0.f) | (q0.w != 0.f) | (q1.x != 0.f) |
                                (q1.y != 0.f) | (q1.z != 0.f) | (q1.w != 0.f) | (q2.x != 0.f) | (q2.y != 0.f) |
                                (q2.z != 0.f) | (q2.w != 0.f) | (q3.x != 0.f) | (q3.y != 0.f) | (q3.z != 0.f) |
                                (q3.w != 0.f) | (q4.x != 0.f);
           if (touched) {
             const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
             gp[0] = z; gp[1] = z; gp[2] = z; gp[3] = z; gp[4] = z;
-          }
-          const float gr[17] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w, q2.x,
-                                q2.y, q2.z, q2.w, q3.x, q3.y, q3.z, q3.w, q4.x};
-          // camera frame (FP32 is enough for the chain rule)
-          float mc[3];
-          mc[0] = fmaf(vw.R[0], f.mx, fmaf(vw.R[1], f.my, fmaf(vw.R[2], f.mz, vw.t[0])));
-          mc[1] = fmaf(vw.R[3], f.mx, fmaf(vw.R[4], f.my, fmaf(vw.R[5], f.mz, vw.t[1])));
-          mc[2] = fmaf(vw.R[6], f.mx, fmaf(vw.R[7], f.my, fmaf(vw.R[8], f.mz, vw.t[2])));
-          float Ur[3], Vr[3], nc[3], U[3], V[3];
-          rot3(vw.R, f.tu, Ur);
-          rot3(vw.R, f.tv, Vr);
-          rot3(vw.R, f.nw, nc);
-          for (int j = 0; j < 3; j++) {
-            U[j] = Ur[j] * f.su;
-            V[j] = Vr[j] * f.sv;
-          }
-          const float flip = dot3(nc, mc) > 0.f ? -1.f : 1.f;
-          for (int j = 0; j < 3; j++) nc[j] *= flip;
-          float av[3], bv[3], nv3[3];
-          cross3(V, mc, av);
-          cross3(mc, U, bv);
-          cross3(U, V, nv3);
-          const float iz = 1.0f / mc[2];
-          const float nn = sqrtf(dot3(nv3, nv3)) * sqrtf(dot3(mc, mc)) * iz;
-          float gU[3] = {0.f, 0.f, 0.f}, gV[3] = {0.f, 0.f, 0.f}, gmc[3] = {0.f, 0.f, 0.f};
-          if (nn > 0.f && isfinite(nn)) {
-            const float iN = 1.0f / nn;
-            const float ifx = vw.ifx, ify = vw.ify;
-            // d/d(rows of adj): the normalisation carries no gradient
-            float ga[3] = {gr[G_P00] * sk * ifx * iN, gr[G_P01] * sk * ify * iN, 0.f};
-            float gb[3] = {gr[G_P10] * sk * ifx * iN, gr[G_P11] * sk * ify * iN, 0.f};
-            const float gS = gr[G_P22] * iN;
-            const float S = dot3(nv3, mc) * iz;
-            float gn[3] = {gr[G_P20] * ifx * iN + gS * mc[0] * iz, gr[G_P21] * ify * iN + gS * mc[1] * iz,
-                           gS * mc[2] * iz};
-            gmc[0] += gS * nv3[0] * iz;
-            gmc[1] += gS * nv3[1] * iz;
-            gmc[2] += gS * nv3[2] * iz - gS * S * iz;
+            const float gr[17] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w, q2.x,
+                                  q2.y, q2.z, q2.w, q3.x, q3.y, q3.z, q3.w, q4.x};
+            // camera frame (FP32 is enough for the chain rule)
+            float mc[3];
+            mc[0] = fmaf(vw.R[0], f.mx, fmaf(vw.R[1], f.my, fmaf(vw.R[2], f.mz, vw.t[0])));
+            mc[1] = fmaf(vw.R[3], f.mx, fmaf(vw.R[4], f.my, fmaf(vw.R[5], f.mz, vw.t[1])));
+            mc[2] = fmaf(vw.R[6], f.mx, fmaf(vw.R[7], f.my, fmaf(vw.R[8], f.mz, vw.t[2])));
+            float Ur[3], Vr[3], nc[3], U[3], V[3];
+            rot3(vw.R, f.tu, Ur);
+            rot3(vw.R, f.tv, Vr);
+            rot3(vw.R, f.nw, nc);
+            for (int j = 0; j < 3; j++) {
+              U[j] = Ur[j] * f.su;
+              V[j] = Vr[j] * f.sv;
+            }
+            const float flip = dot3(nc, mc) > 0.f ? -1.f : 1.f;
+            for (int j = 0; j < 3; j++) nc[j] *= flip;
+            float av[3], bv[3], nv3[3];
+            cross3(V, mc, av);
+            cross3(mc, U, bv);
+            cross3(U, V, nv3);
+            const float iz = 1.0f / mc[2];
+            const float nn = sqrtf(dot3(nv3, nv3)) * sqrtf(dot3(mc, mc)) * iz;
+            float gU[3] = {0.f, 0.f, 0.f}, gV[3] = {0.f, 0.f, 0.f}, gmc[3] = {0.f, 0.f, 0.f};
+            if (nn > 0.f && isfinite(nn)) {
+              const float iN = 1.0f / nn;
+              const float ifx = vw.ifx, ify = vw.ify;
+              // d/d(rows of adj): the normalisation carries no gradient
+              float ga[3] = {gr[G_P00] * sk * ifx * iN, gr[G_P01] * sk * ify * iN, 0.f};
+              float gb[3] = {gr[G_P10] * sk * ifx * iN, gr[G_P11] * sk * ify * iN, 0.f};
+              const float gS = gr[G_P22] * iN;
+              const float S = dot3(nv3, mc) * iz;
+              float gn[3] = {gr[G_P20] * ifx * iN + gS * mc[0] * iz, gr[G_P21] * ify * iN + gS * mc[1] * iz,
+                             gS * mc[2] * iz};
+              gmc[0] += gS * nv3[0] * iz;
+              gmc[1] += gS * nv3[1] * iz;
+              gmc[2] += gS * nv3[2] * iz - gS * S * iz;
+              float t[3];
+              // a = V x mu
+              cross3(mc, ga, t); for (int j = 0; j < 3; j++) gV[j] += t[j];
+              cross3(ga, V, t); for (int j = 0; j < 3; j++) gmc[j] += t[j];
+              // b = mu x U
+              cross3(U, gb, t); for (int j = 0; j < 3; j++) gmc[j] += t[j];
+              cross3(gb, mc, t); for (int j = 0; j < 3; j++) gU[j] += t[j];
+              // n = U x V
+              cross3(V, gn, t); for (int j = 0; j < 3; j++) gU[j] += t[j];
+              cross3(gn, U, t); for (int j = 0; j < 3; j++) gV[j] += t[j];
+            }
+            // projected center and depth
+            gmc[0] += gr[G_CX] * vw.fx * iz;
+            gmc[1] += gr[G_CY] * vw.fy * iz;
+            gmc[2] += -(gr[G_CX] * vw.fx * mc[0] + gr[G_CY] * vw.fy * mc[1]) * iz * iz + gr[G_Z];
+            const float gnc[3] = {gr[G_NX], gr[G_NY], gr[G_NZ]};
+            // pose: d/drho = g_mu_c; d/dphi = sum X x g_X over X in {mu_c, U, V, n_c}
             float t[3];
-            // a = V x mu
-            cross3(mc, ga, t); for (int j = 0; j < 3; j++) gV[j] += t[j];
-            cross3(ga, V, t); for (int j = 0; j < 3; j++) gmc[j] += t[j];
-            // b = mu x U
-            cross3(U, gb, t); for (int j = 0; j < 3; j++) gmc[j] += t[j];
-            cross3(gb, mc, t); for (int j = 0; j < 3; j++) gU[j] += t[j];
-            // n = U x V
-            cross3(V, gn, t); for (int j = 0; j < 3; j++) gU[j] += t[j];
-            cross3(gn, U, t); for (int j = 0; j < 3; j++) gV[j] += t[j];
+            pose[0] = gmc[0]; pose[1] = gmc[1]; pose[2] = gmc[2];
+            cross3(mc, gmc, t); pose[3] += t[0]; pose[4] += t[1]; pose[5] += t[2];
+            cross3(U, gU, t); pose[3] += t[0]; pose[4] += t[1]; pose[5] += t[2];
+            cross3(V, gV, t); pose[3] += t[0]; pose[4] += t[1]; pose[5] += t[2];
+            cross3(nc, gnc, t); pose[3] += t[0]; pose[4] += t[1]; pose[5] += t[2];
+            // back to world
+            float w3[3];
+            rot3T(vw.R, gmc, w3); for (int j = 0; j < 3; j++) gm[j] += w3[j];
+            rot3T(vw.R, gU, w3);
+            gsu += dot3(f.tu, w3);
+            for (int j = 0; j < 3; j++) gtu[j] += f.su * w3[j];
+            rot3T(vw.R, gV, w3);
+            gsv += dot3(f.tv, w3);
+            for (int j = 0; j < 3; j++) gtv[j] += f.sv * w3[j];
+            rot3T(vw.R, gnc, w3);
+            for (int j = 0; j < 3; j++) gnw[j] += flip * w3[j];
+            gop += gr[G_OP];
+            gc[0] += gr[G_R]; gc[1] += gr[G_G]; gc[2] += gr[G_B];
           }
-          // projected center and depth
-          gmc[0] += gr[G_CX] * vw.fx * iz;
-          gmc[1] += gr[G_CY] * vw.fy * iz;
-          gmc[2] += -(gr[G_CX] * vw.fx * mc[0] + gr[G_CY] * vw.fy * mc[1]) * iz * iz + gr[G_Z];
-          const float gnc[3] = {gr[G_NX], gr[G_NY], gr[G_NZ]};
-          // pose: d/drho = g_mu_c; d/dphi = sum X x g_X over X in {mu_c, U, V, n_c}
-          float t[3];
-          pose[0] = gmc[0]; pose[1] = gmc[1]; pose[2] = gmc[2];
-          cross3(mc, gmc, t); pose[3] += t[0]; pose[4] += t[1]; pose[5] += t[2];
-          cross3(U, gU, t); pose[3] += t[0]; pose[4] += t[1]; pose[5] += t[2];
-          cross3(V, gV, t); pose[3] += t[0]; pose[4] += t[1]; pose[5] += t[2];
-          cross3(nc, gnc, t); pose[3] += t[0]; pose[4] += t[1]; pose[5] += t[2];
-          // back to world
-          float w3[3];
-          rot3T(vw.R, gmc, w3); for (int j = 0; j < 3; j++) gm[j] += w3[j];
-          rot3T(vw.R, gU, w3);
-          gsu += dot3(f.tu, w3);
-          for (int j = 0; j < 3; j++) gtu[j] += f.su * w3[j];
-          rot3T(vw.R, gV, w3);
-          gsv += dot3(f.tv, w3);
-          for (int j = 0; j < 3; j++) gtv[j] += f.sv * w3[j];
-          rot3T(vw.R, gnc, w3);
-          for (int j = 0; j < 3; j++) gnw[j] += flip * w3[j];
-          gop += gr[G_OP];
-          gc[0] += gr[G_R]; gc[1] += gr[G_G]; gc[2] += gr[G_B];
         }
       }
+      if (!__any_sync(0xffffffffu, touched)) continue;
       // pose of view v: reduce across the warp when the warp agrees on v
       const int v0 = __shfl_sync(0xffffffffu, v, 0);
       const bool uniform = __all_sync(0xffffffffu, v == v0);
@@ -613,7 +622,7 @@ cudaError_t launch_preprocess_bwd(const splat2d_surfels* S, const Layout& L, con
   A.hdr = reinterpret_cast<const Header*>(ws + L.header);
   A.out = *G;
   A.atomic_params = atomic_params ? 1 : 0;
-  int64_t blocks_cap = (int64_t)sm_count() * 8;
+  int64_t blocks_cap = (int64_t)sm_count() * 24;
   int64_t per = (n_work + blocks_cap - 1) / blocks_cap;
   per = ((per + 255) / 256) * 256;
   if (per < 256) per = 256;
