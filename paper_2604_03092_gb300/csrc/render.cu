@@ -323,9 +323,10 @@ __device__ __forceinline__ int nth_set_bit(uint32_t b, int r) {
   return pos;
 }
 
-// Sum 8 per-lane values over the warp and give every lane all 8 totals
-// (a transposing butterfly: each level halves the values a lane keeps).
-__device__ __forceinline__ void warp_sum8_all(float (&v)[8], int lane) {
+// Sum 8 per-lane values over the warp; lane L returns the total of value
+// (L >> 2) & 7 (a transposing butterfly: each level halves the values a lane
+// keeps).
+__device__ __forceinline__ float warp_sum8(float (&v)[8], int lane) {
 #pragma unroll
   for (int i = 0; i < 4; i++) {
     const bool up = lane & 16;
@@ -348,8 +349,11 @@ __device__ __forceinline__ void warp_sum8_all(float (&v)[8], int lane) {
   }
   v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
   v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-  // lane L now holds the total of value index (L >> 2) & 7
-  const float t0 = v[0];
+  return v[0];
+}
+// ... and every lane gets all 8 totals.
+__device__ __forceinline__ void warp_sum8_all(float (&v)[8], int lane) {
+  const float t0 = warp_sum8(v, lane);
 #pragma unroll
   for (int k = 0; k < 8; k++) v[k] = __shfl_sync(0xffffffffu, t0, k << 2);
 }
@@ -374,7 +378,7 @@ __device__ __forceinline__ float warp_scan_add(float x, int lane) {
 
 // Per-pixel state of the forward while it is handed between warps.
 struct FwdState {
-  float T, C0, C1, C2, D, N0, N1, N2, Ds;
+  float T, C0, C1, C2, D, N0, N1, N2, Ds;  // k_render_tail takes C0..Ds as an array
   uint32_t last, done;
 };
 
@@ -663,7 +667,7 @@ __global__ void __launch_bounds__(TW* TH, 3) k_render_fwd(const RenderArgs A) {
 // Issue-bound (71% of the issue slots on 4 keyframes x 4 views); the blending
 // pass keeps 17% of its lanes busy where many keyframes overlap, 41% on one.
 // With k_render_tail, against k_render_fwd for all of it: 24 keyframes x 24
-// views at 512x384 16.3 -> 12.2 ms; one keyframe x 8 views 557 -> 465 us.
+// views at 512x384 16.3 -> 11.9 ms; one keyframe x 8 views 557 -> 465 us.
 constexpr int WARPS = 4;       // warps per CTA of the warp-per-tile forward
 constexpr int FW_STRIDE = 33;  // floats per pixel row of the alpha table
 // (pixel, entry) pairs per 32 pixels (of 1024) that make a chunk dense: two
@@ -1088,7 +1092,11 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
 // one's are composited, and each pixel's entries as bit masks, from the rects
 // by a transpose.  8 keyframes in one view, both forward kernels, against two
 // warps per tile and a record gather by lane: 300 tiles 1200 -> 1052 us, 3072
-// tiles 467 -> 434; 24 keyframes x 24 views 12.5 -> 12.2 ms.
+// tiles 467 -> 434; 24 keyframes x 24 views 12.5 -> 12.2 ms.  With many tiles
+// by shared memory (76% of its pipe): four lanes keep each of a pixel's eight
+// sums, for all lanes all of them, and colours, normals and depths are read for
+// the entries that contribute: 8 keyframes x 8 views 319 -> 296 us, 24 x 24
+// forward 12.12 -> 11.95 ms.
 template <int CHUNK>
 struct TailSmem {
   static constexpr int W = CHUNK / 32;
@@ -1208,20 +1216,21 @@ __global__ void __launch_bounds__(CHUNK, 768 / CHUNK) k_render_tail(const Render
         }
         __syncwarp();
         const float fx = (float)(tx0 + (pth & 7)) + 0.5f, fy = (float)(ty0 + (pth >> 3)) + 0.5f;
-        FwdState st = S.st[pth];
-        float acc[8] = {st.C0, st.C1, st.C2, st.D, st.N0, st.N1, st.N2, st.Ds};
-        float tt = st.T;
-        uint32_t lst = st.last;
+        // the eight sums lie after T; four lanes keep one of them
+        float* sums = &S.st[pth].C0;
+        float acc = sums[(lane >> 2) & 7], tt = S.st[pth].T;
+        uint32_t lst = S.st[pth].last;
         bool dn = false;
         for (int g = 0; g < nrel && !dn; g += 32) {
           const bool has = g + lane < nrel;
           const int j = has ? (int)S.list[wid][g + lane] : 0;
           const float4* rec = S.raw + j * REC_F4;
-          const float4 f2 = rec[2], f3 = rec[3], f4 = rec[4];
           Pair e;
+          float4 f2;
           float alpha = 0.f;
           if (has) {
             const float4 f0 = rec[0];
+            f2 = rec[2];
             const float2 cl = unpack_half2_scaled(__float_as_uint(f0.z));
             eval_pair(make_float4(f0.x, f0.y, cl.x, cl.y), rec[1], make_float4(f2.x, f2.y, f2.z, f0.w), fx, fy,
                       P.lp_scale, P.alpha_max, e);
@@ -1243,6 +1252,7 @@ __global__ void __launch_bounds__(CHUNK, 768 / CHUNK) k_render_tail(const Render
             float vals[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             float zpair = 0.f;
             if (contrib) {
+              const float4 f3 = rec[3], f4 = rec[4];
               zpair = pair_depth(e, f4.y, f2.z, P.depth_ray);
               vals[0] = w * f2.w; vals[1] = w * f3.x; vals[2] = w * f3.y;
               vals[3] = w * zpair;
@@ -1251,20 +1261,20 @@ __global__ void __launch_bounds__(CHUNK, 768 / CHUNK) k_render_tail(const Render
             if constexpr (DIST) {
               // depth sum in front of each pair: the pixel's so far, then the group's own terms before it
               const float wz = vals[3];
-              const float Bb = acc[3] + (warp_scan_add(wz, lane) - wz);
+              const float Bb = __shfl_sync(0xffffffffu, acc, 12) + (warp_scan_add(wz, lane) - wz);
               vals[7] = contrib ? 2.f * w * (zpair * (1.f - Tb) - Bb) : 0.f;
             }
-            warp_sum8_all(vals, lane);
-#pragma unroll
-            for (int q = 0; q < 8; q++) acc[q] += vals[q];
+            acc += warp_sum8(vals, lane);
             if (contrib) atomicOr(&S.bits[j >> 5][pth], 1u << (j & 31));
             lst = (uint32_t)(base + __shfl_sync(0xffffffffu, j, 31 - __clz(cb)) + 1);
           }
           dn = stopb != 0u;
           tt = dn ? __shfl_sync(0xffffffffu, Tb, sl) : __shfl_sync(0xffffffffu, Ta, 31);
         }
+        if ((lane & 3) == 0) sums[lane >> 2] = acc;
         if (lane == 0) {
-          S.st[pth] = FwdState{tt, acc[0], acc[1], acc[2], acc[3], acc[4], acc[5], acc[6], acc[7], lst, 0u};
+          S.st[pth].T = tt;
+          S.st[pth].last = lst;
           if (!dn) S.apix[cur ^ 1][atomicAdd(&S.nact[cur ^ 1], 1)] = (uint16_t)pth;
         }
         __syncwarp();
