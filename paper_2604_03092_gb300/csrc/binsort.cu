@@ -498,8 +498,9 @@ __device__ unsigned long long* block_radix_reg(unsigned long long* a, unsigned l
   unsigned long long* src = a;
   unsigned long long* dst = b;
   auto digit = [&](unsigned long long key, int shift) -> uint32_t {
-    const unsigned long long dk = (unsigned long long)((uint32_t)(key >> 32) - dmin);
-    const unsigned long long kk = ishift < 0 ? dk : ((dk << ishift) | (unsigned long long)((uint32_t)key - imin));
+    const uint32_t dk = (uint32_t)(key >> 32) - dmin;
+    if (ishift < 0) return (dk >> (shift + lsb)) & 0xffu;  // the depth part: no 64-bit shifts
+    const unsigned long long kk = ((unsigned long long)dk << ishift) | (unsigned long long)((uint32_t)key - imin);
     return (uint32_t)(kk >> (shift + lsb)) & 0xffu;
   };
   int first = 0;
@@ -950,17 +951,15 @@ struct SegClass {
 template <int NWARPS, int ITEMS, bool LAST>
 // The bucket is sorted in place in one shared buffer (each radix pass holds
 // its keys in registers between its loads and its scatter, with block
-// barriers in between), so the 1025..4096, 4097..6144 and 6145..8192 classes
-// (41, 57 and 73 KB of shared memory) run 3 CTAs per SM under a 42-register
-// bound: their keys spill, but the third CTA hides more of the barrier waits
-// (binning 10.01 -> 9.82 ms for the first class, 9.82 -> 9.62 ms for the
-// second, on the 32-keyframe submap; sorting the 6145..8192 buckets there
-// instead of in the 1024-thread class at one CTA per SM: 9.63 -> 9.37 ms, and
-// 9.46 ms at 2 CTAs per SM without the spills).  The 257..2048 class (256
-// threads, 21 KB) runs 6 CTAs per SM, which matters where buckets are short
-// (64 uneven submaps: binning 11.62 -> 11.35 ms for taking the 1025..2048
-// buckets out of the 512-thread class).
-__global__ void __launch_bounds__(NWARPS * 32, NWARPS == 16 ? 3 : (NWARPS == 8 ? 6 : 1)) k_tile_sort(const SegArgs A) {
+// barriers in between).  Bound by issue and by the barriers, so more CTAs per
+// SM pay even where their keys spill: the 257..2048 class (256 threads, 21 KB
+// of shared memory) runs 7 under a 36-register bound, the 2049..4096 class (512
+// threads, 41 KB) 4 under 32, and the 4097..6144 and 6145..8192 classes (57 and
+// 73 KB) 3 under 40, which their shared memory allows (under 32 as well: 24 x
+// 24 5556 us).  Against 6 and 3 CTAs, and digits by 64-bit shifts: binning 840
+// -> 785 us (8 keyframes x 8 views), 5734 -> 5538 (24 x 24), 731 -> 724 (12
+// uneven submaps); 5 or 4 CTAs of the first class 861, 868, 8 of them 789.
+__global__ void __launch_bounds__(NWARPS * 32, NWARPS == 16 ? (ITEMS == 8 ? 4 : 3) : (NWARPS == 8 ? 7 : 1)) k_tile_sort(const SegArgs A) {
   using C = SegClass<NWARPS, ITEMS>;
   extern __shared__ __align__(16) unsigned char smem[];
   unsigned long long* sa = reinterpret_cast<unsigned long long*>(smem);
