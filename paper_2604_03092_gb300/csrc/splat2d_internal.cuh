@@ -250,6 +250,15 @@ __device__ __forceinline__ float2 unpack_half2_scaled(uint32_t u) {
   return make_float2(f.x * (1.0f / 65536.0f), f.y * (1.0f / 65536.0f));
 }
 
+// Whether the step has failed (an exceeded instance capacity leaves no valid
+// lists), the same answer for all of a CTA.  In the checked build an index
+// check may set the status while other CTAs are still starting; threads that
+// read it one by one could part, and the ones that stay would wait for the
+// others at a barrier or work on an item that nobody has taken.  Every thread
+// calls it, before the CTA's first item.  It reads through L2, for kernels
+// that start beside the one before.
+__device__ __forceinline__ bool step_failed(const Header* hdr) { return __syncthreads_or(__ldcg(&hdr->status) != 0); }
+
 // Leaves a persistent kernel's work queue: the last CTA to leave sets it, the
 // count of those that left and `more` back to zero for the kernel's next
 // launch.  Every thread calls it, once, after the CTA's last item.
