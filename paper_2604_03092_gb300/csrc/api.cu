@@ -20,16 +20,15 @@ std::atomic<uint64_t>& launch_counter() {
 void count_launches(int n) { launch_counter().fetch_add((uint64_t)n); }
 
 int sm_count() {
-  static int cached[64] = {0};
+  static PerDevice cache;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-  if (dev < 0 || dev >= 64) dev = 0;
-  if (!cached[dev]) {
-    int n = 0;
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    cached[dev] = n > 0 ? n : 1;
-  }
-  return cached[dev];
+  const int n = cache.get(dev, [dev] {
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+  });
+  return n < 1 ? 1 : n;
 }
 
 static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }

@@ -1011,13 +1011,8 @@ template <int NWARPS, int ITEMS, bool LAST>
 static cudaError_t launch_tile_sort_class(const SegArgs& S, cudaStream_t st) {
   using C = SegClass<NWARPS, ITEMS>;
   auto k = k_tile_sort<NWARPS, ITEMS, LAST>;
-  static int per_sm = -1;
-  if (per_sm < 0) {
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, C::THREADS, C::SMEM);
-    if (per_sm < 1) per_sm = 1;
-  }
-  return launch_chained(k, per_sm * sm_count(), C::THREADS, C::SMEM, st, S);
+  static PerDevice resident;
+  return launch_chained(k, resident_ctas(resident, k, C::THREADS, C::SMEM), C::THREADS, C::SMEM, st, S);
 }
 
 // Count, scan, scatter (which also lists the tiles by size class) and the
@@ -1090,13 +1085,9 @@ cudaError_t launch_bin_tiles(const Layout& L, const RastParams& P, char* ws, cud
     S.queue = queues + c;
     switch (c) {
       case 0: {
-        static int per_sm = -1;
-        if (per_sm < 0) {
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_sort_warp, WS_WARPS * 32, 0);
-          if (per_sm < 1) per_sm = 1;
-        }
-        const int64_t most = (L.T + WS_WARPS - 1) / WS_WARPS;
-        e = launch_chained(k_tile_sort_warp, (int)min64(most, (int64_t)per_sm * sm_count()), WS_WARPS * 32, 0, st, S);
+        static PerDevice resident;
+        const int grid = persistent_grid(resident, k_tile_sort_warp, WS_WARPS * 32, 0, (L.T + WS_WARPS - 1) / WS_WARPS);
+        e = launch_chained(k_tile_sort_warp, grid, WS_WARPS * 32, 0, st, S);
         break;
       }
       case 1: e = launch_tile_sort_class<8, 8, false>(S, st); break;

@@ -2004,59 +2004,29 @@ static RenderArgs make_args(const Layout& L, const RastParams& P, char* ws, cons
   return A;
 }
 
-template <typename K>
-static int persistent_grid(K kernel, int threads, size_t smem, int64_t work) {
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
-  if (per_sm < 1) per_sm = 1;
-  int64_t g = (int64_t)per_sm * sm_count();
-  if (g > work) g = work;
-  return (int)(g < 1 ? 1 : g);
-}
-
 template <int TW, int TH, int CHUNK, bool DIST>
 static cudaError_t run_fwd_k(const RenderArgs& A, cudaStream_t st) {
   auto k = k_render_fwd<TW, TH, CHUNK, DIST>;
   constexpr size_t smem = sizeof(FwdSmem<TW * TH, CHUNK>);
-  static int grid = -1;
-  static int64_t grid_T = -1;
-  if (grid < 0) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (grid < 0 || grid_T != A.T) {
-    grid = persistent_grid(k, TW * TH, smem, A.T);
-    grid_T = A.T;
-  }
-  return launch_chained(k, grid, TW * TH, smem, st, A);
+  static PerDevice resident;
+  return launch_chained(k, persistent_grid(resident, k, TW * TH, smem, A.T), TW * TH, smem, st, A);
 }
-// One warp-per-tile launch: NP = 2 pixels per lane, or 1 (two items per tile).
-template <int NP, typename K>
-static cudaError_t run_warp_kernel(K k, size_t smem, const RenderArgs& A, int64_t& grid_T, int& grid, cudaStream_t st) {
-  const int64_t items = NP == 2 ? A.T : 2 * A.T;
-  if (grid < 0) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (grid < 0 || grid_T != A.T) {
-    grid = persistent_grid(k, WARPS * 32, smem, (items + WARPS - 1) / WARPS);
-    grid_T = A.T;
-  }
-  return launch_chained(k, grid, WARPS * 32, smem, st, A);
-}
+// The warp-per-tile kernel: NP = 2 pixels per lane, or 1 (two items per tile).
 template <int NP, bool RAY, bool DIST>
 static cudaError_t run_fwd_warp(const RenderArgs& A, cudaStream_t st) {
-  static int grid = -1;
-  static int64_t grid_T = -1;
-  return run_warp_kernel<NP>(k_render_fwd_warp<NP, RAY, DIST>, sizeof(FwdWarpSmem<NP, RAY>) * WARPS, A, grid_T, grid,
-                             st);
+  auto k = k_render_fwd_warp<NP, RAY, DIST>;
+  constexpr size_t smem = sizeof(FwdWarpSmem<NP, RAY>) * WARPS;
+  static PerDevice resident;
+  const int64_t items = NP == 2 ? A.T : 2 * A.T;
+  const int grid = persistent_grid(resident, k, WARPS * 32, smem, (items + WARPS - 1) / WARPS);
+  return launch_chained(k, grid, WARPS * 32, smem, st, A);
 }
 template <int CHUNK, bool DIST>
 static cudaError_t run_tail(const RenderArgs& A, cudaStream_t st) {
   auto k = k_render_tail<CHUNK, DIST>;
   constexpr size_t smem = sizeof(TailSmem<CHUNK>);
-  static int grid = -1;
-  static int64_t grid_T = -1;
-  if (grid < 0) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (grid < 0 || grid_T != A.T) {
-    grid = persistent_grid(k, CHUNK, smem, A.T);
-    grid_T = A.T;
-  }
-  return launch_chained(k, grid, CHUNK, smem, st, A);
+  static PerDevice resident;
+  return launch_chained(k, persistent_grid(resident, k, CHUNK, smem, A.T), CHUNK, smem, st, A);
 }
 template <int NP>
 static cudaError_t run_fwd_tiles8(const RenderArgs& A, cudaStream_t st) {
@@ -2071,14 +2041,8 @@ template <int TW, int TH, int CHUNK, bool DIST>
 static cudaError_t run_bwd_k(const RenderArgs& A, cudaStream_t st) {
   auto k = k_render_bwd<TW, TH, CHUNK, DIST>;
   constexpr size_t smem = sizeof(BwdSmem<TW * TH, CHUNK, DIST>);
-  static int grid = -1;
-  static int64_t grid_T = -1;
-  if (grid < 0) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (grid < 0 || grid_T != A.T) {
-    grid = persistent_grid(k, TW * TH, smem, A.T);
-    grid_T = A.T;
-  }
-  return launch_chained(k, grid, TW * TH, smem, st, A);
+  static PerDevice resident;
+  return launch_chained(k, persistent_grid(resident, k, TW * TH, smem, A.T), TW * TH, smem, st, A);
 }
 template <int TW, int TH, int CHUNK>
 static cudaError_t run_bwd(const RenderArgs& A, cudaStream_t st) {
@@ -2088,24 +2052,15 @@ static cudaError_t run_bwd(const RenderArgs& A, cudaStream_t st) {
 template <int TW, int TH>
 static cudaError_t run_max_error(const RenderArgs& A, const float* err, uint32_t* max_err, cudaStream_t st) {
   auto k = k_max_error<TW, TH>;
-  static int grid = -1;
-  static int64_t grid_T = -1;
-  if (grid < 0 || grid_T != A.T) {
-    grid = persistent_grid(k, TW * TH, 0, A.T);
-    grid_T = A.T;
-  }
-  k<<<grid, TW * TH, 0, st>>>(A, err, max_err);
+  static PerDevice resident;
+  k<<<persistent_grid(resident, k, TW * TH, 0, A.T), TW * TH, 0, st>>>(A, err, max_err);
   count_launches(1);
   return cudaGetLastError();
 }
 
 static cudaError_t run_max_error_ranked(const RenderArgs& A, const float* err, uint32_t* max_err, cudaStream_t st) {
-  static int grid = -1;
-  static int64_t grid_T = -1;
-  if (grid < 0 || grid_T != A.T) {
-    grid = persistent_grid(k_max_error_ranked, ME_WARPS * 32, 0, A.T);
-    grid_T = A.T;
-  }
+  static PerDevice resident;
+  const int grid = persistent_grid(resident, k_max_error_ranked, ME_WARPS * 32, 0, A.T);
   return launch_chained(k_max_error_ranked, grid, ME_WARPS * 32, 0, st, A, err, max_err);
 }
 

@@ -9,6 +9,7 @@
 #include <atomic>
 
 #include "splat2d.h"
+#include "per_device.h"
 
 namespace s2d {
 
@@ -189,6 +190,28 @@ inline cudaError_t launch_chained(void (*kernel)(K...), int grid, int threads, s
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, K(args)...);
   count_launches(1);
   return e;
+}
+
+// CTAs of a kernel that the current device holds at once; on a device's first
+// call the kernel is allowed its dynamic shared memory there.  `cache`: the
+// kernel's own.
+template <typename K>
+inline int resident_ctas(PerDevice& cache, K kernel, int threads, size_t smem) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  const int n = cache.get(dev, [&] {
+    if (smem && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return 0;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess) return 0;
+    return per_sm * sm_count();
+  });
+  return n < 1 ? sm_count() : n;
+}
+// ... of a persistent kernel with `work` items.
+template <typename K>
+inline int persistent_grid(PerDevice& cache, K kernel, int threads, size_t smem, int64_t work) {
+  return (int)max64(1, min64(work, resident_ctas(cache, kernel, threads, smem)));
 }
 
 // Error-free transformations (Knuth's TwoSum; the FMA-based exact product).
