@@ -144,7 +144,7 @@ template <bool SCATTER>
 __global__ void __launch_bounds__(256) k_tile_bin(const TileBinArgs A) {
   chain_release();
   chain_wait();
-  if (SCATTER && step_failed(A.hdr)) return;
+  if (SCATTER && step_failed(A.hdr->status)) return;
   if (SCATTER) classify_tiles(A.ranges, A.T, A.class_list, A.class_count, A.order_count);
   const int lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -917,7 +917,7 @@ __global__ void __launch_bounds__(WS_WARPS * 32, 6) k_tile_sort_warp(const SegAr
   __shared__ __align__(16) WarpSortSmem s_sort[WS_WARPS];
   chain_wait();
   chain_release();  // after the wait: the next class starts without one (see k_tile_sort)
-  if (step_failed(A.hdr)) return;
+  if (step_failed(A.hdr->status)) return;
   order_tiles(A.ranges, A.T, A.order_count, A.order_cursor, A.order);
   const int lane = threadIdx.x & 31;
   WarpSortSmem& S = s_sort[threadIdx.x >> 5];
@@ -977,7 +977,7 @@ __global__ void __launch_bounds__(NWARPS * 32, NWARPS == 16 ? (ITEMS == 8 ? 4 : 
   // them start, and the wait for the class before comes last.  Until then
   // what the scatter wrote is read through L2.
   chain_release();
-  const uint32_t n_tiles = step_failed(A.hdr) ? 0u : __ldcg(A.list_count);
+  const uint32_t n_tiles = step_failed(__ldcg(&A.hdr->status)) ? 0u : __ldcg(A.list_count);
   for (;;) {
     if (threadIdx.x == 0) s_q = atomicAdd(A.queue, 1u);
     __syncthreads();

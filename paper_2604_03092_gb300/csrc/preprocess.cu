@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(256, 3) k_preprocess_bwd(const PreBwdArgs A) {
   chain_release();
   chain_wait();
   // a failed binning (instance capacity exceeded): nothing was accumulated
-  if (step_failed(A.hdr)) return;
+  if (step_failed(A.hdr->status)) return;
   const int64_t wlo = (int64_t)blockIdx.x * A.per_block;
   const int64_t whi = min(wlo + A.per_block, A.n_work);
   if (wlo >= whi) return;

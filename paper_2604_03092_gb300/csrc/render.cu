@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(TW* TH, 3) k_render_fwd(const RenderArgs A) {
   chain_release();
   chain_wait();
   // a failed binning (instance capacity exceeded) leaves no valid lists
-  if (step_failed(A.hdr)) return;
+  if (step_failed(A.hdr->status)) return;
   for (;;) {
     if (threadIdx.x == 0) S.item = (int)atomicAdd(&A.hdr->queue_fwd, 1u);
     __syncthreads();
@@ -866,7 +866,7 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
   chain_release();
   chain_wait();
   // a failed binning (instance capacity exceeded) leaves no valid lists
-  if (step_failed(A.hdr)) return;
+  if (step_failed(A.hdr->status)) return;
   for (;;) {
     uint32_t item = 0;
     const int half = NP == 1 ? (threadIdx.x >> 5) & 1 : 0;
@@ -1123,7 +1123,7 @@ __global__ void __launch_bounds__(CHUNK, 768 / CHUNK) k_render_tail(const Render
   chain_release();
   chain_wait();
   // a failed binning (instance capacity exceeded) leaves no valid lists
-  if (step_failed(A.hdr)) return;
+  if (step_failed(A.hdr->status)) return;
   const int n_items = (int)A.hdr->n_tails;
   if (n_items == 0) return;
   for (;;) {
@@ -1463,7 +1463,7 @@ __global__ void __launch_bounds__(TW* TH, (TW * TH == 64) ? (CHUNK <= 64 ? 16 : 
   chain_release();
   chain_wait();
   // a failed binning (instance capacity exceeded) leaves no valid lists
-  if (step_failed(A.hdr)) return;
+  if (step_failed(A.hdr->status)) return;
   const bool want_n = A.d_normal != nullptr;  // normal terms only when their gradient is asked for
   // The pixel at tile-local (x, y) is laid out by warp (x + 3y) mod NW -- a
   // diagonal interleave, so every warp's 32 pixels spread over the whole tile
@@ -1837,7 +1837,7 @@ __global__ void __launch_bounds__(TW* TH) k_max_error(const RenderArgs A, const 
   __shared__ int s_item;
   __shared__ uint32_t s_top;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (step_failed(A.hdr)) return;
+  if (step_failed(A.hdr->status)) return;
   for (;;) {
     if (threadIdx.x == 0) s_item = (int)atomicAdd(&A.hdr->queue_aux, 1u);
     __syncthreads();
@@ -1910,7 +1910,7 @@ __global__ void __launch_bounds__(ME_WARPS * 32) k_max_error_ranked(const Render
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   chain_release();
   chain_wait();
-  if (step_failed(A.hdr)) return;
+  if (step_failed(A.hdr->status)) return;
   for (;;) {
     if (tid == 0) s_item = (int)atomicAdd(&A.hdr->queue_aux, 1u);
     __syncthreads();

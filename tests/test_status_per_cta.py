@@ -18,13 +18,15 @@ def _code(path):
 
 
 def test_kernels_read_the_status_through_step_failed():
-    uses, callers = [], 0
+    direct, through = [], 0
     for name in sorted(os.listdir(CSRC)):
         code = _code(os.path.join(CSRC, name))
-        callers += len(re.findall(r"\bstep_failed\(A\.hdr\)", code))
-        uses += [(name, m.group(0).strip()) for m in re.finditer(r"[^\n]*hdr->status[^\n]*", code)]
-    allowed = (r"bool step_failed\(.*__syncthreads_or\(.*hdr->status", r"hdr->status = SPLAT2D_ERR_CAPACITY;",
-               r"atomicCAS\(.*&hdr->status")
-    assert [u for u in uses if not any(re.search(a, u[1]) for a in allowed)] == []
+        code, n = re.subn(r"\bstep_failed\((?:A\.hdr->status|__ldcg\(&A\.hdr->status\))\)", "", code)
+        through += n
+        direct += [(name, m.group(0).strip()) for m in re.finditer(r"[^\n]*hdr->status[^\n]*", code)]
+    writes = (r"hdr->status = SPLAT2D_ERR_CAPACITY;", r"atomicCAS\(.*&hdr->status")
+    assert [u for u in direct if not any(re.search(w, u[1]) for w in writes)] == []
     # scatter, the two bucket sorts, the chain rule and the six kernels of render.cu
-    assert callers == 10
+    assert through == 10
+    body = _code(os.path.join(CSRC, "splat2d_internal.cuh")).split("bool step_failed(", 1)[1].split("\n}", 1)[0]
+    assert re.search(r"#ifdef S2D_CHECKS\s+return __syncthreads_or\(status != 0\);", body)
