@@ -237,7 +237,13 @@ struct PinnedHeader {
     return p;
   }
   ~PinnedHeader() {
-    if (p && owner == getpid()) cudaFreeHost(p);
+    if (!p || owner != getpid()) return;
+    // a thread may end while another one captures a graph: a call that frees
+    // memory would end that capture with an error, but in this mode
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    cudaFreeHost(p);
+    cudaThreadExchangeStreamCaptureMode(&mode);
   }
 };
 
