@@ -302,8 +302,8 @@ static int preprocess_checked(const splat2d_config* cfg, const splat2d_surfels* 
   std::memcpy(tables.data() + (L.views - L.header), H.views.data(), sizeof(DView) * H.views.size());
   if (!H.groups.empty())
     std::memcpy(tables.data() + (L.groups - L.header), H.groups.data(), sizeof(DGroup) * H.groups.size());
-  if (launch_setup(tables.data(), table_bytes, L, w, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
-  if (launch_preprocess(surfels, L, make_params(cfg), w, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+  if (launch_setup(tables.data(), table_bytes, L, w, st) != cudaSuccess) return cuda_error();
+  if (launch_preprocess(surfels, L, make_params(cfg), w, st) != cudaSuccess) return cuda_error();
   return SPLAT2D_OK;
 }
 
@@ -334,7 +334,7 @@ int splat2d_bin_sort(const splat2d_config* cfg, const splat2d_problem* prob, voi
   if (rc) return rc;
   if (launch_bin_tiles(L, make_params(cfg), static_cast<char*>(ws), reinterpret_cast<cudaStream_t>(stream)) !=
       cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
+    return cuda_error();
   return SPLAT2D_OK;
 }
 
@@ -343,7 +343,7 @@ static int render_fwd_checked(const splat2d_config* cfg, const Layout& L, char* 
   const uint32_t* vals = reinterpret_cast<const uint32_t*>(w + (final_sorted_buffer(L) ? L.vals1 : L.vals0));
   if (launch_render_fwd(L, make_params(cfg), cfg->chunk, w, vals, rgb, depth, normal, alpha, dist, st) !=
       cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
+    return cuda_error();
   return SPLAT2D_OK;
 }
 
@@ -370,7 +370,7 @@ int splat2d_forward(const splat2d_config* cfg, const splat2d_problem* prob, cons
   char* w = static_cast<char*>(ws);
   rc = preprocess_checked(cfg, surfels, L, H, w, st);
   if (rc) return rc;
-  if (launch_bin_tiles(L, make_params(cfg), w, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+  if (launch_bin_tiles(L, make_params(cfg), w, st) != cudaSuccess) return cuda_error();
   return render_fwd_checked(cfg, L, w, rgb, depth, normal, alpha, dist, st);
 }
 
@@ -390,7 +390,7 @@ int splat2d_render_bwd_tiles_dist(const splat2d_config* cfg, const splat2d_probl
   const uint32_t* vals = reinterpret_cast<const uint32_t*>(w + (final_sorted_buffer(L) ? L.vals1 : L.vals0));
   if (launch_render_bwd(L, make_params(cfg), cfg->bwd_chunk ? cfg->bwd_chunk : cfg->chunk, w, vals, d_rgb,
                         d_depth, d_normal, d_alpha, d_dist, st) != cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
+    return cuda_error();
   return SPLAT2D_OK;
 }
 
@@ -412,7 +412,7 @@ int splat2d_preprocess_bwd(const splat2d_config* cfg, const splat2d_problem* pro
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (launch_preprocess_bwd(surfels, L, make_params(cfg), static_cast<char*>(ws), grads, L.groups_overlap, st) !=
       cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
+    return cuda_error();
   return SPLAT2D_OK;
 }
 
@@ -426,7 +426,7 @@ int splat2d_max_error(const splat2d_config* cfg, const splat2d_problem* prob, vo
   char* w = static_cast<char*>(ws);
   const uint32_t* vals = reinterpret_cast<const uint32_t*>(w + (final_sorted_buffer(L) ? L.vals1 : L.vals0));
   if (launch_max_error(L, make_params(cfg), cfg->chunk, w, vals, err, max_err, st) != cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
+    return cuda_error();
   return SPLAT2D_OK;
 }
 
@@ -438,7 +438,7 @@ int splat2d_accum_gate(const float* alpha, int64_t n, float tau, uint32_t* keep_
   if (n > 0 && (!alpha || !keep_idx || !tmp)) return SPLAT2D_ERR_INVALID_ARG;
   if (n > 0 && tmp_bytes < accum_gate_tmp_size(n)) return SPLAT2D_ERR_WORKSPACE_TOO_SMALL;
   if (launch_accum_gate(alpha, n, tau, keep_idx, n_keep, tmp, reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
+    return cuda_error();
   return SPLAT2D_OK;
 }
 
@@ -459,7 +459,7 @@ int splat2d_voxelize(const splat2d_surfels* in, int32_t width, int32_t height, f
   }
   if (launch_voxelize(*in, width, height, tau_d, *out, out_block, n_out, tmp, reinterpret_cast<cudaStream_t>(stream)) !=
       cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
+    return cuda_error();
   return SPLAT2D_OK;
 }
 
@@ -467,7 +467,7 @@ int splat2d_sim3_apply(int64_t n, float* means, float* quats, float* scales, con
                        const int32_t* index, splat2d_stream stream) {
   if (n < 0 || (n > 0 && !sim3)) return SPLAT2D_ERR_INVALID_ARG;
   if (launch_sim3(n, means, quats, scales, sim3, index, reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
+    return cuda_error();
   return SPLAT2D_OK;
 }
 
@@ -499,12 +499,12 @@ int splat2d_stats(const void* ws, splat2d_stats_t* out, splat2d_stream stream) {
   Header* dst = pinned.get();
   Header h;
   if (dst) {
-    if (cudaMemcpyAsync(dst, ws, sizeof(Header), cudaMemcpyDeviceToHost, st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
-    if (cudaStreamSynchronize(st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+    if (cudaMemcpyAsync(dst, ws, sizeof(Header), cudaMemcpyDeviceToHost, st) != cudaSuccess) return cuda_error();
+    if (cudaStreamSynchronize(st) != cudaSuccess) return cuda_error();
     h = *dst;
   } else {
-    if (cudaStreamSynchronize(st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
-    if (cudaMemcpy(&h, ws, sizeof(Header), cudaMemcpyDeviceToHost) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+    if (cudaStreamSynchronize(st) != cudaSuccess) return cuda_error();
+    if (cudaMemcpy(&h, ws, sizeof(Header), cudaMemcpyDeviceToHost) != cudaSuccess) return cuda_error();
   }
   std::memset(out, 0, sizeof(*out));
   out->status = h.status;
@@ -545,15 +545,15 @@ int splat2d_sort_pairs(uint64_t* keys, uint32_t* vals, int64_t n, int key_bits, 
   uint32_t* v1 = reinterpret_cast<uint32_t*>(t + align256(sizeof(uint64_t) * n));
   uint32_t* hist = reinterpret_cast<uint32_t*>(t + align256(sizeof(uint64_t) * n) + align256(sizeof(uint32_t) * n));
   const int nb = std::min(SORT_MAX_BLOCKS, 4 * sm_count());
-  if (cudaMemsetAsync(hist + 256 * (size_t)nb, 0, 256 * sizeof(uint32_t), st) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+  if (cudaMemsetAsync(hist + 256 * (size_t)nb, 0, 256 * sizeof(uint32_t), st) != cudaSuccess) return cuda_error();
   int fb = 0;
   if (launch_sort(keys, vals, k1, v1, nullptr, n, key_bits, hist, nb, &fb, st) != cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
+    return cuda_error();
   if (fb) {
     if (cudaMemcpyAsync(keys, k1, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-      return SPLAT2D_ERR_CUDA;
+      return cuda_error();
     if (cudaMemcpyAsync(vals, v1, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-      return SPLAT2D_ERR_CUDA;
+      return cuda_error();
   }
   return SPLAT2D_OK;
 }

@@ -71,7 +71,7 @@ extern "C" int splat2d_sort_pairs_noalloc(uint64_t* keys, uint32_t* vals, int64_
   if (n == 0) return SPLAT2D_OK;
   if (!keys || !vals) return SPLAT2D_ERR_INVALID_ARG;
   void* base = nullptr;
-  if (scratch_address(&base) != cudaSuccess) return SPLAT2D_ERR_CUDA;
+  if (scratch_address(&base) != cudaSuccess) return cuda_error();
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* t = static_cast<char*>(base);
   uint64_t* k1 = reinterpret_cast<uint64_t*>(t);
@@ -81,15 +81,15 @@ extern "C" int splat2d_sort_pairs_noalloc(uint64_t* keys, uint32_t* vals, int64_
   if (nb > SORT_MAX_BLOCKS) nb = SORT_MAX_BLOCKS;
   // the array keeps the previous call's contents: the digit totals must start at zero
   if (cudaMemsetAsync(hist + 256 * (size_t)nb, 0, 256 * sizeof(uint32_t), st) != cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
+    return cuda_error();
   int fb = 0;
   if (launch_sort(keys, vals, k1, v1, nullptr, n, key_bits, hist, nb, &fb, st) != cudaSuccess)
-    return SPLAT2D_ERR_CUDA;
+    return cuda_error();
   if (fb) {
     if (cudaMemcpyAsync(keys, k1, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-      return SPLAT2D_ERR_CUDA;
+      return cuda_error();
     if (cudaMemcpyAsync(vals, v1, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-      return SPLAT2D_ERR_CUDA;
+      return cuda_error();
   }
   return SPLAT2D_OK;
 }

@@ -161,6 +161,13 @@ cudaError_t launch_preprocess_bwd(const splat2d_surfels* S, const Layout& L, con
 int sm_count();
 void count_launches(int n);  // host-side tally of kernels enqueued
 
+// What a call returns where a CUDA call failed, which takes that failure out of
+// the runtime's last error: launches read it, and would report it once more.
+inline int cuda_error() {
+  cudaGetLastError();
+  return SPLAT2D_ERR_CUDA;
+}
+
 // ---------------------------------------------------------------------------
 // Device helpers
 // ---------------------------------------------------------------------------
