@@ -161,7 +161,7 @@ typedef struct {
   int64_t needed_capacity;     /* instances the last binning needed */
   int64_t n_instances;         /* instances binned and sorted */
   int64_t n_visible;           /* visible (view, surfel) pairs */
-  int64_t fwd_pairs_evaluated; /* (pixel, surfel) pairs whose alpha the forward computed */
+  int64_t fwd_pairs_evaluated; /* (pixel, surfel) pairs up to each pixel's stop: alphas the forward needs */
   int64_t fwd_pairs_blended;   /* ... of which blended */
   int64_t bwd_pairs_evaluated; /* (pixel, surfel) pairs the reverse pass recomputed */
   int64_t bwd_pairs_blended;   /* ... of which carried gradient */
