@@ -816,10 +816,11 @@ struct PixelSums {
 };
 
 // Blends the entries of `todo` (ascending) into one pixel; returns those
-// blended (all, or those before the first that would take T below t_min, `stop`).
+// blended (all, or those before the first that would take T below t_min, whose
+// number goes to the padding of the pixel's row).
 template <int NP, bool RAY, bool DIST>
-__device__ __forceinline__ uint32_t blend_pixel(const FwdWarpSmem<NP, RAY>& S, int pix, uint32_t todo, float px,
-                                                float py, float t_min, PixelSums<DIST>& s, bool& done, int& stop) {
+__device__ __forceinline__ uint32_t blend_pixel(FwdWarpSmem<NP, RAY>& S, int pix, uint32_t todo, float px, float py,
+                                                float t_min, PixelSums<DIST>& s, bool& done) {
   uint32_t k = todo;
   while (k) {
     const int e = __ffs(k) - 1;
@@ -828,7 +829,7 @@ __device__ __forceinline__ uint32_t blend_pixel(const FwdWarpSmem<NP, RAY>& S, i
     const float Tn = __fmul_rn(s.T, __fsub_rn(1.f, alpha));
     if (Tn < t_min) {
       done = true;
-      stop = e;
+      S.alpha[pix * FW_STRIDE + 32] = __int_as_float(e);
       return todo & ((1u << e) - 1u);
     }
     k &= k - 1;
@@ -973,16 +974,33 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
       }
       __syncwarp();
       const uint32_t pairs = count_bits<NP>(m);
-      n_eval += pairs;
       uint32_t bl[NP];  // entries blended at this lane's pixels
-      int stop[NP];     // ... and the entry at which a pixel stops
 #pragma unroll
-      for (int h = 0; h < NP; h++) {
-        bl[h] = 0u;
-        stop[h] = 32;
-      }
+      for (int h = 0; h < NP; h++) bl[h] = 0u;
+      // Takes the pairs behind the stops of this chunk off the count, whose alphas
+      // have been computed all the same: fwd_pairs_evaluated is the work that any
+      // schedule has.  The stops lie in the table's padding: as registers they
+      // cost spills.  With whole tiles a dense chunk counts as it goes.  Against
+      // counting all pairs of the chunk: 24 keyframes x 24 views 12.65 -> 12.48 ms,
+      // 8 keyframes x 8 views with distortion 2080 -> 2115 us, one keyframe in
+      // 192 tiles 183 -> 188.
+      auto settle = [&]() {
+        uint32_t gone[NP];
+#pragma unroll
+        for (int h = 0; h < NP; h++) gone[h] = live_px[h] & __ballot_sync(0xffffffffu, done[h]);
+        if (!P.stats || !any_bits<NP>(gone)) return;
+        const uint32_t rect = ok ? S.rect(lane) : 0u;
+#pragma unroll
+        for (int h = 0; h < NP; h++) {
+          if (!gone[h]) continue;
+          const uint32_t in = warp_transpose_bits(rect_pixels(rect, h), lane);
+          if ((gone[h] >> lane) & 1u)
+            n_eval -= __popc(in & ~((2u << __float_as_int(S.alpha[(lane + 32 * h) * FW_STRIDE + 32])) - 1u));
+        }
+      };
       if (__reduce_add_sync(0xffffffffu, pairs) >= FW_DENSE * NP) {
         // ---- dense chunk: every lane walks every entry at its pixels -----------
+        int stop = 31;  // NP = 1
 #pragma unroll 2
         for (int e = 0; e < count; e++) {
           const float4* rec = raw + e * REC_F4;
@@ -994,11 +1012,13 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
 #pragma unroll
           for (int h = 0; h < NP; h++) {
             const uint32_t on = (__shfl_sync(0xffffffffu, m[h], e) >> lane) & 1u;
-            if (!on || done[h] || pr.alpha[h] < P.alpha_min) continue;
+            if (!on || done[h]) continue;
+            if (NP == 2) n_eval++;
+            if (pr.alpha[h] < P.alpha_min) continue;
             const float Tn = __fmul_rn(ps[h].T, __fsub_rn(1.f, pr.alpha[h]));
             if (Tn < P.t_min) {
               done[h] = true;
-              stop[h] = e;
+              if (NP == 1) stop = e;
               continue;
             }
             const float zp = RAY && pr.obj[h] ? f4.y * f2.z * pr.rc[h] : f4.y;  // see pair_depth
@@ -1007,8 +1027,15 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
             bl[h] |= 1u << e;
           }
         }
+        if constexpr (NP == 1) {
+          n_eval += pairs;
+          __syncwarp();  // the records have been read
+          if (done[0]) S.alpha[lane * FW_STRIDE + 32] = __int_as_float(stop);
+          settle();
+        }
       } else {
         // ---- pass 1: alphas, an entry per lane ---------------------------------
+        n_eval += pairs;
         uint32_t kept[NP];  // pixels where this entry's alpha is at least alpha_min
 #pragma unroll
         for (int h = 0; h < NP; h++) kept[h] = 0u;
@@ -1056,21 +1083,8 @@ __global__ void __launch_bounds__(WARPS * 32, RAY ? 5 : 6) k_render_fwd_warp(con
         __syncwarp();
 #pragma unroll
         for (int h = 0; h < NP; h++)
-          bl[h] = blend_pixel<NP, RAY, DIST>(S, lane + 32 * h, todo[h], px, h ? py1 : py0, P.t_min, ps[h], done[h],
-                                             stop[h]);
-      }
-      // The pairs behind a pixel's stop don't count, although their alphas have
-      // been computed: fwd_pairs_evaluated is the work that any schedule has.
-      // (24 keyframes x 24 views 12.64 -> 12.73 ms, one keyframe x 8 443.6 ->
-      // 449 us; with the rects read back from the copy 12.83, 452.)
-      if (P.stats && __any_sync(0xffffffffu, (stop[0] & stop[NP - 1]) < 32)) {
-        const uint32_t rect = ok ? S.rect(lane) : 0u;
-#pragma unroll
-        for (int h = 0; h < NP; h++) {
-          if (!__any_sync(0xffffffffu, stop[h] < 32)) continue;
-          const uint32_t in = warp_transpose_bits(rect_pixels(rect, h), lane);
-          if (stop[h] < 32) n_eval -= __popc(in & ~((2u << stop[h]) - 1u));
-        }
+          bl[h] = blend_pixel<NP, RAY, DIST>(S, lane + 32 * h, todo[h], px, h ? py1 : py0, P.t_min, ps[h], done[h]);
+        settle();
       }
 #pragma unroll
       for (int h = 0; h < NP; h++) {
