@@ -953,13 +953,13 @@ template <int NWARPS, int ITEMS, bool LAST>
 // its keys in registers between its loads and its scatter, with block
 // barriers in between).  Bound by issue and by the barriers, so more CTAs per
 // SM pay even where their keys spill: the 257..2048 class (256 threads, 21 KB
-// of shared memory) runs 7 under a 36-register bound, the 2049..4096 class (512
-// threads, 41 KB) 4 under 32, and the 4097..6144 and 6145..8192 classes (57 and
-// 73 KB) 3 under 40, which their shared memory allows (under 32 as well: 24 x
-// 24 5556 us).  Against 6 and 3 CTAs, and digits by 64-bit shifts: binning 840
-// -> 785 us (8 keyframes x 8 views), 5734 -> 5538 (24 x 24), 731 -> 724 (12
-// uneven submaps); 5 or 4 CTAs of the first class 861, 868, 8 of them 789.
-__global__ void __launch_bounds__(NWARPS * 32, NWARPS == 16 ? (ITEMS == 8 ? 4 : 3) : (NWARPS == 8 ? 7 : 1)) k_tile_sort(const SegArgs A) {
+// of shared memory) runs 8 with 32 registers a thread, the 2049..4096 class (512
+// threads, 41 KB) 4 with 32, and the 4097..6144 and 6145..8192 classes (57 and
+// 73 KB) 3 with 40, which their shared memory allows (with 32 as well: 24 x 24
+// 5556 us).  Against 6 and 3 CTAs, and digits by 64-bit shifts: binning 840 ->
+// 785 us (8 keyframes x 8 views), 5734 -> 5538 (24 x 24), 731 -> 724 (12 uneven
+// submaps); 5 or 4 CTAs of the first class 861, 868.
+__global__ void __launch_bounds__(NWARPS * 32, NWARPS == 16 ? (ITEMS == 8 ? 4 : 3) : (NWARPS == 8 ? 8 : 1)) k_tile_sort(const SegArgs A) {
   using C = SegClass<NWARPS, ITEMS>;
   extern __shared__ __align__(16) unsigned char smem[];
   unsigned long long* sa = reinterpret_cast<unsigned long long*>(smem);

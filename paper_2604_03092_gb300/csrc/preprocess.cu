@@ -302,7 +302,7 @@ __device__ __forceinline__ uint32_t project_one(const PreArgs& A, const DView& v
 // shifts, here and in the binning, for divisions by a size that is known at
 // run time only, and colours read where the surfel is visible: 48 keyframes in
 // one view 226 -> 189 us, 8 keyframes x 8 views 330 -> 308 (binning 852 ->
-// 840), 24 x 24 2395 -> 2221 (5861 -> 5784).
+// 840), 24 x 24 2395 -> 2222 (5861 -> 5772).
 // ONE_VIEW: no surfel is in two views.  Most of a map is then outside its
 // view, and the others are told from center and size, before the rotation is
 // read: 48 keyframes in one view 187 -> 154 us.  With more views a surfel most
@@ -402,7 +402,7 @@ constexpr int kPoseSlots = 64;  // per-block pose accumulators (views)
 // Bound by the latency of the gradient records and by issue.  A record that no
 // pixel touched, its gradient zero, adds nothing and skips the chain rule, a
 // warp of them the pose sums too.  Three CTAs per SM of 80 registers, for four
-// of 64 that spill; up to 24 blocks per SM, for 8, which left the last ones
+// of 64 that spill more; up to 24 blocks per SM, for 8, which left the last ones
 // uneven: one keyframe x 8 views 107 -> 92 us, 8 x 8 558 -> 486, 24 x 24 3481
 // -> 3141, 12 uneven submaps 440 -> 417 (48 blocks 94, 492, 3129, 420, without
 // the skip 92, 492, 3157, 422; each block adds its pose sums in FP32).

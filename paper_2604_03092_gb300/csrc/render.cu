@@ -675,12 +675,22 @@ constexpr int FW_STRIDE = 33;  // floats per pixel row of the alpha table
 // it; 275 and 450 were slower on keyframes.
 constexpr uint32_t FW_DENSE = 350;
 // Up to this many tiles per SM a warp takes half a tile: twice the warps, and
-// a shorter chain per chunk, where the tiles are too few for whole ones to
-// keep the SM's 24 warps busy.  Whole against half, one keyframe in one view:
-// 300 tiles 186 / 144 us, 1200 88 / 80, 1938 88 / 98, 3072 97 / 117, 4800
-// 117 / 133; 8 keyframes: 300 tiles 1349 / 1052, 1200 511 / 401, 1938 429 /
-// 423, 3072 434 / 440, 4800 409 / 497; 2688 tiles of large surfels (dense
-// chunks) 148 / 106.
+// a shorter chain per chunk, for about a fifth more work in all.  That pays where
+// the longest lists decide when the last warp is done, so up to some 8 tiles
+// per SM always, beyond as long as the load lies on some of the tiles.  Whole /
+// half tiles, us, by tiles:
+//                          1200        1900        2494        3185        4800
+//   1 keyframe          82 /  72    82 /  96    88 / 106    93 / 111   107 / 125
+//   3 keyframes        200 / 161   175 / 193   171 / 189   181 / 221   213 / 262
+//   8 keyframes        562 / 453   473 / 403   422 / 392   411 / 406   399 / 488
+//   32 keyframes      2267 /1911  1857 /1516  1519 /1209  1369 /1028  1124 / 882
+//   20 K surfels       130 /  98   128 /  95   131 /  93   133 / 100
+//   60 K small ones     95 /  76    93 /  69    98 /  66   101 /  66   (4200) 106 / 80
+// No tile count is right for all: this one costs a few keyframes up to 19% at
+// 1500 to 2700 tiles and many, or a map in the image's middle, up to 50% at 2700
+// to 6000; 4.6% in the mean of 132 such scenes.  The longest list against the
+// mean load tells them apart, but is known on the device only: a launch of both
+// with one of them idle costs uniform scenes the 3 to 7% it gains on others.
 constexpr int FW_WHOLE_TILES_PER_SM = 18;
 
 template <int NP>
