@@ -661,13 +661,13 @@ __global__ void __launch_bounds__(TW* TH, 3) k_render_fwd(const RenderArgs A) {
 // pixels in the tile are more even in number than the entries of a pixel,
 // which the depth order concentrates in a band of the tile; the evaluation
 // reads no shared memory; and the pairs below alpha_min (40% of them) never
-// reach the pass that blends: 6.9 warp instructions per evaluated pair against
-// 10.2.  A chunk whose rects cover a third of the pixels or more is walked by
+// reach the pass that blends: with k_render_tail 8.0 warp instructions per
+// evaluated pair against 12.7 (8 keyframes x 8 views).  A chunk whose rects cover a third of the pixels or more is walked by
 // all lanes together instead.
 // Issue-bound (71% of the issue slots on 4 keyframes x 4 views); the blending
 // pass keeps 17% of its lanes busy where many keyframes overlap, 41% on one.
 // With k_render_tail, against k_render_fwd for all of it: 24 keyframes x 24
-// views at 512x384 16.3 -> 11.9 ms; one keyframe x 8 views 557 -> 465 us.
+// views at 512x384 16.3 -> 11.8 ms; one keyframe x 8 views 557 -> 460 us.
 constexpr int WARPS = 4;       // warps per CTA of the warp-per-tile forward
 constexpr int FW_STRIDE = 33;  // floats per pixel row of the alpha table
 // (pixel, entry) pairs per 32 pixels (of 1024) that make a chunk dense: two
